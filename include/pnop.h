@@ -64,7 +64,10 @@ enum {
  *     the FP32 rate on this GPU.
  * Everything else (the radial banded solves, the influence and flux
  * corrections, the base flow, the stage combinations, energies and inner
- * products) stays FP64.  PNOP_FP64 (0) is FP64 throughout. */
+ * products) stays FP64.  PNOP_FP64 (0) is FP64 throughout.  In every precision
+ * the banded solves run in 64-bit block-floating integer arithmetic, which
+ * rounds below FP64 arithmetic, where a grid's factors fit it (all unstretched
+ * grids of 21 radial points or more), else in FP64. */
 enum { PNOP_FP64 = 0, PNOP_MIXED = 1, PNOP_DF = 2, PNOP_MIXED_DF = 3 };
 
 /* Grid.  nr radial points (>= 9); ntheta, nz nominal azimuthal/axial sizes,

@@ -3,14 +3,16 @@
 // replaces Eq. 2.9-2.11).
 //
 // Spectral fields are FP64 complex, layout [c][j][m + M][k].  Everything here
-// is FP64: the curl and base-flow terms, and everything radial (banded
-// matvecs, banded LU solves, influence and flux corrections).  The theta/z
+// carries FP64 values: the curl and base-flow terms, and everything radial
+// (banded matvecs, banded solves, influence and flux corrections).  The theta/z
 // transforms are in transforms.cu.  Every kernel also serves batched launches:
 // it finds its batch entry in one grid dimension and offsets its field
 // pointers and per-request tables by that entry's slot (see Geo).
 #include "dev_common.cuh"
 #include "dev_df.cuh"
+#include "dev_x64.cuh"
 #include "kernels.hpp"
+#include "setup.hpp"
 
 #include <algorithm>
 #include <string>
@@ -685,8 +687,7 @@ __global__ void k_stage_div(Geo g, const double2* __restrict__ F, double2* __res
 // copy.  Each of the 2 kSK threads sweeps the real or the imaginary part of one
 // system (the matrices are real).  Terms are accumulated oldest first, so the
 // dependence from one row to the next is a single FMA.
-constexpr int kRC = 8;        // rows per staged chunk
-constexpr int kRegRows = 64;  // grids up to this many radial points keep their columns in registers
+constexpr int kRC = 8;  // rows per staged chunk
 
 __device__ __forceinline__ void cp_async16(void* sm, const void* gm) {
     const unsigned a = (unsigned)__cvta_generic_to_shared(sm);
@@ -800,7 +801,7 @@ __global__ void __launch_bounds__(2 * kSK) k_band_solve(Geo g, const double* __r
         }
         __syncthreads();
     }
-    if (WALL && k0 + sy < g.nk) {  // wall partials of the tentative velocity (as in k_band_solve_reg)
+    if (WALL && k0 + sy < g.nk) {  // wall partials of the tentative velocity (as in k_band_solve_x)
         usub = moved(usub, off);
         const double* us = usub ? reinterpret_cast<const double*>(usub) + comp : nullptr;
         double* P = pw + ((((size_t)slot * 3 + v) * g.nm + im) * g.nk + (k0 + sy)) * 2 + comp;
@@ -836,163 +837,450 @@ __global__ void __launch_bounds__(2 * kSK) k_band_solve(Geo g, const double* __r
     }
 }
 
-// The same two-sweep solve with each thread's column held in registers
-// (grids of at most MAXR radial points; the launch bound of six blocks per SM
-// keeps the register count at 168, which holds the column without spills).  The column stays in x[0..MAXR): the
-// forward sweep reads its lower neighbours and the backward sweep its upper
-// neighbours straight from registers (every index is a compile-time constant
-// after unrolling), so no shared-memory round trip sits on the dependent
-// chain of a row; shared memory holds only the staged coefficient rows.  The
-// arithmetic and its order are those of k_band_solve: the results are the
-// same to the last bit (up to the sign of zero).
-template <int NL, int NU, bool DIAG1, int MAXR, bool WALL>
-__global__ void __launch_bounds__(2 * kSK, 6) k_band_solve_reg(Geo g, const double* __restrict__ fac, size_t fac_stride,
-                                                      double2* __restrict__ X, const double2* __restrict__ add,
-                                                      int helm, int zero_row0, double* __restrict__ pw,
-                                                      const double2* __restrict__ usub) {
+// The solve in block-floating integer arithmetic (dev_x64.cuh), the path of
+// every table whose multipliers fit the fixed-point format (the host decides,
+// see setup.hpp; the FP64 kernel above serves the others).  The FP64 pipe bounds
+// that kernel at 52 us for the 24,192 Helmholtz systems of 64x64x256 (9
+// instructions of 77 cycles per row and real part) and its row-to-row chain at
+// 36 us for the 8,064 pressure systems; here each is bound by integer issue and
+// by a chain of half the length, since a system is taken from both ends at once
+// (table and factorisation: setup.hpp).  Both directions are the same sweeps
+// with the multipliers gathered by row or by column:
+//   A x = b:    N r = b (inwards),    M x = r (outwards)
+//   A^T x = b:  M^T v = b (inwards),  N^T x = D^-1 v (outwards).
+// A row takes four multipliers, and the rows that meet the one-sided wall
+// stencils four more.  Rows go in chunks of four.  A chunk's right-hand sides
+// and the window of the last four results share one exponent, chosen so that
+// the largest has its top bit at 53 or above (a rounding is at most 2^-54 of
+// it, where FP64 arithmetic rounds at 2^-53 of every partial sum) and all stay
+// below 2^60; a chunk whose results outgrow that (a warp vote on their
+// magnitudes, which cannot wrap: one row adds at most a factor 1 + kFxRowSum)
+// is redone with a coarser unit.  Between the sweeps a row stays in fixed point
+// (in place of its right-hand side, each lane reading what it wrote).
+//
+// A block is one (component, m) and 16 consecutive k, a warp per side, lane
+// pairs holding the real and imaginary parts; multipliers stream through the
+// warp's own shared memory with cp.async.  The two warps meet once, at the middle.
+// Measured against the FP64 kernels that served these solves before (64x64x256,
+// ncu): pressure 36.8 -> 23.7 us, Helmholtz with the wall partials 71.2 -> 49.4
+// us, the transposed pair 37.5 + 74.8 -> 23.7 + 51.5 us; at 32x32x64 25.5 -> 14.8
+// us per solve.  Half as many rows per FP64 chain (the same sweeps in FP64, two-
+// sided) measured 33 and 96 us, and tiles split between the integer and the FP64
+// form 34 and 61 us: the FP64 pipe is the slower partner either way.
+constexpr int kXR = 4;         // rows per chunk
+constexpr int kXK = 16;        // systems of a block
+constexpr int kXChunks = 96;   // most chunks of a side
+struct XShape {
+    int chunks[2], pad, in[2], out[2], mid[2], wall, tile;  // of FxShape
+};
+
+// The window of a sweep: the results of the last chunk (slot i: its row i) and,
+// near the wall, the values only the wall rows read, in units of 2^E.
+struct XWin {
+    xdig w[4], x[4];
+    int gw, gx;  // high-digit magnitudes
+    int E;
+    bool wall;  // x in use
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i].h = w[i].l = x[i].h = x[i].l = 0;
+        gw = gx = 0;
+        E = kXZero;
+        wall = false;
+    }
+    __device__ __forceinline__ void coarsen(int d) {  // unit times 2^d
+        E += d;
+        const int r = min(max(d, 0), 63), l = min(max(-d, 0), 63);
+        gw = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            w[i] = x_split((x_join(w[i]) >> r) << l);
+            gw |= x_mag(w[i]);
+        }
+        if (wall) {
+            gx = 0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                x[i] = x_split((x_join(x[i]) >> r) << l);
+                gx |= x_mag(x[i]);
+            }
+        }
+    }
+    // makes room for right-hand sides that need units of at least 2^e
+    __device__ __forceinline__ void align(int e) {
+        const int mx = gw | gx;
+        if (!__any_sync(0xffffffffu, e > E || mx >= (1 << 26) || (mx < (1 << 21) && e < E - 6))) return;
+        int low = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) low |= w[i].h | w[i].l | x[i].h | x[i].l;
+        const int top = mx ? 63 - __clz(mx) : 31;  // bit the largest value may reach
+        coarsen(max(low ? top - 55 : kXZero, e + 4 - E));
+    }
+};
+
+// one double, or nothing (a predicate instead of a branch)
+__device__ __forceinline__ double ld_if(const double* p, bool on) {
+    double v;
+    asm volatile("{\n .reg .pred q;\n setp.ne.s32 q, %2, 0;\n mov.f64 %0, 0d0000000000000000;\n"
+                 " @q ld.global.f64 %0, [%1];\n}" : "=d"(v) : "l"(p), "r"((int)on) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_if(double* p, double v, bool on) {
+    asm volatile("{\n .reg .pred q;\n setp.ne.s32 q, %2, 0;\n @q st.global.f64 [%0], %1;\n}"
+                 :: "l"(p), "d"(v), "r"((int)on) : "memory");
+}
+
+// What a warp of the solver works on, and its streams: a side of the 16 systems
+// of a block, multipliers into shared memory a chunk ahead, right-hand sides
+// (on the way back: intermediate values) into registers a chunk ahead.
+struct XSide {
+    int2 (*buf)[kXR * 5 * kXK];  // two chunks of multipliers
+    const int2* mid;             // this side's half of the middle
+    const int2 *tin, *tout;      // tables
+    int side, lane, n, pad;
+    bool on;          // the lane's k exists
+    double* xp;       // the lane's value of position p: xp[p step] (positions below pad do not exist)
+    const double* ad;  // the same of a field to add, or null
+    ptrdiff_t step;
+    double nx[kXR], an[kXR];
+
+    // chunk t of the sweep sequence: inwards 0 .. n - 1, outwards n - 2 .. 0
+    __device__ __forceinline__ void stage(int t) {
+        int2* dst = buf[t & 1] + 2 * lane;
+        if (t < n) {
+            const int2* src = tin + t * (kXR * 4 * kXK) + 2 * lane;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) cp_async16(dst + 64 * i, src + 64 * i);
+        } else if (t < 2 * n - 1) {
+            const int2* src = tout + (2 * n - 2 - t) * (kXR * 5 * kXK) + 2 * lane;
+#pragma unroll
+            for (int i = 0; i < 5; ++i) cp_async16(dst + 64 * i, src + 64 * i);
+        }
+        cp_async_commit();
+    }
+    __device__ __forceinline__ void ready() {  // the chunk staged before the last one has arrived
+        cp_async_wait1();
+        __syncwarp();
+    }
+    __device__ __forceinline__ void load(int t) {
+        const double* q = xp + t * kXR * step;
+        const int first = t ? 0 : pad;
+#pragma unroll
+        for (int r = 0; r < kXR; ++r) nx[r] = ld_if(q + r * step, on && r >= first);
+    }
+    __device__ __forceinline__ void load_add(int t) {
+        const double* q = ad + t * kXR * step;
+        const int first = t ? 0 : pad;
+#pragma unroll
+        for (int r = 0; r < kXR; ++r) an[r] = ld_if(q + r * step, on && r >= first);
+    }
+    __device__ __forceinline__ void store(int t, const double (&v)[kXR]) {
+        double* q = xp + t * kXR * step;
+        const int first = t ? 0 : pad;
+#pragma unroll
+        for (int r = 0; r < kXR; ++r) st_if(q + r * step, v[r], on && r >= first);
+    }
+    // results of chunk t, with what is to be added to them; x9: rows 0..8 for the wall partials
+    __device__ __forceinline__ void finish(int t, double (&v)[kXR], bool zero0, double (*x9)[32]) {
+        if (x9 && side == 0 && t < 3) {
+#pragma unroll
+            for (int r = 0; r < kXR; ++r)
+                if (t * kXR + r < 9) x9[t * kXR + r][lane] = v[r];
+        }
+        if (zero0 && side == 0 && t == 0) v[0] = 0.0;
+        if (ad) {
+#pragma unroll
+            for (int r = 0; r < kXR; ++r) v[r] += an[r];
+            if (t > 0) load_add(t - 1);
+        }
+        store(t, v);
+    }
+};
+
+// The two sweeps of one side in integer arithmetic.
+template <bool TRANS, bool WALL>
+__device__ __forceinline__ void solve_fixed(XSide& a, const int2* TX, int sh0, int helm, int zero_row0,
+                                            int2 (*ex)[kXR][32], int2 (*exu)[32], double (*x9)[32]) {
+    const int kk = a.lane >> 1, n = a.n, side = a.side, lane = a.lane;
+    XWin q;
+    q.clear();
+    const long long half = x_half();
+    auto wall = [&](int i) {  // the four further products of wall row i
+        const int2* c = TX + i * 4 * kXK;
+        return x_dot4(__ldg(c), q.x[0], __ldg(c + kXK), q.x[1], __ldg(c + 2 * kXK), q.x[2], __ldg(c + 3 * kXK), q.x[3],
+                      half);
+    };
+    int mxb = 0;  // largest high word (sign cleared) of the column
+    double b0 = 0.0;
+    short Es[kXChunks];  // units of the chunks between the sweeps
+    for (int t = 0; t < n; ++t) {  // inwards
+        a.stage(t + 1);
+        double b[kXR];
+#pragma unroll
+        for (int r = 0; r < kXR; ++r) b[r] = a.nx[r];
+        if (t + 1 < n) a.load(t + 1);
+        a.ready();
+        const int4* C = reinterpret_cast<const int4*>(a.buf[t & 1]) + kk;
+        if (t == 0 && side == 0) {
+            b0 = b[0];
+            if (!TRANS) {  // column 0 of N: its value enters the window times 2^sh0
+                const int h = __double2hiint(b0), m = h & 0x7FFFFFFF;
+                if (m > 0xFFFFF) b[0] = __hiloint2double(h + sh0 * (1 << 20), __double2loint(b0));
+                if (m >= 0x7FF00000 - sh0 * (1 << 20)) mxb = 0x7FF00000;
+            }
+        }
+        int mb = 0;
+#pragma unroll
+        for (int r = 0; r < kXR; ++r) mb = max(mb, __double2hiint(b[r]) & 0x7FFFFFFF);
+        mxb = max(mxb, mb);
+        if (TRANS && side == 0 && t == 1) {  // rows 5..8 also read v_0..v_3
+#pragma unroll
+            for (int i = 0; i < 4; ++i) q.x[i] = q.w[i];
+            q.gx = q.gw;
+            q.wall = true;
+        }
+        q.align((mb >> 20) - kXTop);
+        xdig nd[kXR];
+        int mg;
+        for (int tries = 0; tries < 4; ++tries) {
+            const xunit u = x_unit(q.E);
+            mg = 0;
+#pragma unroll
+            for (int r = 0; r < kXR; ++r) {
+                auto win = [&](int i) { return r + i < 4 ? q.w[(r + i) & 3] : nd[(r + i) & 3]; };  // position p - 4 + i
+                const int4 c01 = C[(r * 2) * kXK], c23 = C[(r * 2 + 1) * kXK];
+                long long sum = x_dot4(make_int2(c01.x, c01.y), win(0), make_int2(c01.z, c01.w), win(1),
+                                       make_int2(c23.x, c23.y), win(2), make_int2(c23.z, c23.w), win(3), half);
+                if (TRANS && side == 0 && ((t == 1 && r > 0) || (t == 2 && r == 0))) sum += wall(t == 2 ? 3 : r - 1);
+                nd[r] = x_split(x_load(b[r], u) + sum);
+                mg |= x_mag(nd[r]);
+            }
+            if (!__any_sync(0xffffffffu, mg >= (1 << 28))) break;
+            q.coarsen(6);
+        }
+        q.gw = mg;
+#pragma unroll
+        for (int r = 0; r < kXR; ++r) {
+            q.w[r] = nd[r];
+            b[r] = __hiloint2double(nd[r].h, nd[r].l);  // digits, for the way back
+        }
+        if (t + 1 < n) a.store(t, b);
+        Es[t] = (short)q.E;
+        if (TRANS && side == 0 && t == 2) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) q.x[i].h = q.x[i].l = 0;
+            q.gx = 0;
+            q.wall = false;
+        }
+        __syncwarp();
+    }
+    // the middle: this side's four rows of S^-1 (or its transpose) times both
+    // sides' right-hand sides, in the coarser of their units
+#pragma unroll
+    for (int r = 0; r < kXR; ++r) ex[side][r][lane] = make_int2(q.w[r].l, q.w[r].h);
+    exu[side][lane] = make_int2(q.E, mxb);
+    a.load(n - 2);
+    __syncthreads();
+    const int2 ou = exu[side ^ 1][lane];
+    // infinities and NaN anywhere in a column reach every row of a solve
+    const int nan = max(mxb, ou.y) >= 0x7FF00000 ? 0x7FF80000 : 0;
+    long long nv[kXR];
+    {
+        xdig o[kXR];
+        const int E = max(q.E, ou.x), da = min(E - q.E, 63), db = min(E - ou.x, 63);
+#pragma unroll
+        for (int r = 0; r < kXR; ++r) {
+            const int2 t = ex[side ^ 1][r][lane];
+            o[r].l = t.x;
+            o[r].h = t.y;
+            o[r] = x_split(x_join(o[r]) >> db);
+            q.w[r] = x_split(x_join(q.w[r]) >> da);
+        }
+        const int4* G = reinterpret_cast<const int4*>(a.mid) + kk;
+#pragma unroll
+        for (int r = 0; r < kXR; ++r) {
+            const int4 c0 = G[(r * 4) * kXK], c1 = G[(r * 4 + 1) * kXK], c2 = G[(r * 4 + 2) * kXK], c3 = G[(r * 4 + 3) * kXK];
+            nv[r] = x_dot4(make_int2(c0.x, c0.y), q.w[0], make_int2(c0.z, c0.w), q.w[1], make_int2(c1.x, c1.y), q.w[2],
+                           make_int2(c1.z, c1.w), q.w[3], half) +
+                    x_dot4(make_int2(c2.x, c2.y), o[0], make_int2(c2.z, c2.w), o[1], make_int2(c3.x, c3.y), o[2],
+                           make_int2(c3.z, c3.w), o[3], half);
+        }
+        q.clear();
+        q.E = E + a.mid[32 * kXK + kk].x;
+#pragma unroll
+        for (int r = 0; r < kXR; ++r) {
+            q.w[r] = x_split(nv[r]);
+            q.gw |= x_mag(q.w[r]);
+        }
+    }
+    __syncwarp();
+    if (a.ad) a.load_add(n - 1);
+    for (int c = n - 1; c >= 0; --c) {  // outwards: the middle's results first, then a chunk at a time
+        if (c < n - 1) {
+            const int t = 2 * n - 2 - c;
+            a.stage(t + 1);
+            int2 y[kXR];
+#pragma unroll
+            for (int r = 0; r < kXR; ++r) y[r] = make_int2(__double2loint(a.nx[r]), __double2hiint(a.nx[r]));
+            if (c > 0) a.load(c - 1);
+            a.ready();
+            const int4* C = reinterpret_cast<const int4*>(a.buf[t & 1]) + kk;
+            const int2* Cd = a.buf[t & 1] + kXR * 4 * kXK + kk;
+            // D^-1 y, at most 62 bits: 1/D is D' 2^(s - 60), s + 128 the low byte
+            // of D'; the rows of a chunk share s except in the first one
+            long long z[kXR];
+            int mz = 0, mr[kXR], sr[kXR];
+#pragma unroll
+            for (int r = 0; r < kXR; ++r) {
+                const int2 D = Cd[r * kXK];
+                xdig yd;
+                yd.l = y[r].x;
+                yd.h = y[r].y;
+                z[r] = x_prod<60>(D, yd, 4 * half);
+                mr[r] = x_mag(x_split(z[r]));
+                mz |= mr[r];
+                sr[r] = D.x & 0xFF;
+            }
+            int ez = Es[c] - 128 + sr[0], e = ez + (mz ? 63 - __clz(mz) : 31) - 59;
+            if (c == 0) {  // to a common unit
+                int top = kXZero;
+#pragma unroll
+                for (int r = 0; r < kXR; ++r) {
+                    // y_0 was carried times 2^sh0 (direct), or row 0 is summed in units of 2^-sh0 (transposed)
+                    sr[r] += Es[c] - 128 - (r == 0 && side == 0 ? sh0 : 0);
+                    top = max(top, sr[r] + (mr[r] ? 63 - __clz(mr[r]) : 31));
+                }
+                e = ez = top - 59;
+#pragma unroll
+                for (int r = 0; r < kXR; ++r) z[r] = x_move(z[r], ez - sr[r]);
+            }
+            if (!TRANS && side == 0 && c == 1) {  // rows 3..0 also read x_5..x_8
+                q.x[3] = q.w[0];
+                q.gx = q.gw;
+                q.wall = true;
+            }
+            if (!TRANS && side == 0 && c == 0) {
+#pragma unroll
+                for (int i = 0; i < 3; ++i) q.x[i] = q.w[i + 1];
+                q.gx |= q.gw;
+            }
+            q.align(e);
+            xdig nd[kXR];
+            int mg;
+            for (int tries = 0; tries < 4; ++tries) {
+                const int d = q.E - ez, right = min(max(d, 0), 63), left = min(max(-d, 0), 63);
+                mg = 0;
+#pragma unroll
+                for (int r = kXR - 1; r >= 0; --r) {
+                    auto win = [&](int i) { return r + i >= 4 ? q.w[(r + i) & 3] : nd[(r + i) & 3]; };  // position p + i
+                    const int4 c12 = C[(r * 2) * kXK], c34 = C[(r * 2 + 1) * kXK];
+                    long long sum = x_dot4(make_int2(c34.z, c34.w), win(4), make_int2(c34.x, c34.y), win(3),
+                                           make_int2(c12.z, c12.w), win(2), make_int2(c12.x, c12.y), win(1), half);
+                    if (!TRANS && side == 0 && c == 0) sum += wall(r);
+                    nv[r] = ((z[r] >> right) << left) + sum;
+                    nd[r] = x_split(nv[r]);
+                    mg |= x_mag(nd[r]);
+                }
+                if (!__any_sync(0xffffffffu, mg >= (1 << 28))) break;
+                q.coarsen(6);
+            }
+            q.gw = mg;
+#pragma unroll
+            for (int r = 0; r < kXR; ++r) q.w[r] = nd[r];
+        }
+        int nz = 0;
+#pragma unroll
+        for (int r = 0; r < kXR; ++r) nz |= q.w[r].h | q.w[r].l;
+        const bool far = __any_sync(0xffffffffu, nz && (q.E < -1000 || q.E > 900));
+        double res[kXR];
+#pragma unroll
+        for (int r = 0; r < kXR; ++r) {
+            const int Er = TRANS && side == 0 && r == 0 && c == 0 ? q.E + sh0 : q.E;
+            res[r] = far ? x_store_any(nv[r], Er, nan) : x_store(nv[r], Er, nan);
+        }
+        // the Dirichlet row is the unit row: exactly its right-hand side
+        if (!TRANS && helm && side == 0 && c == 0 && !nan) res[0] = b0;
+        a.finish(c, res, zero_row0, WALL ? x9 : nullptr);
+        __syncwarp();
+    }
+}
+
+template <bool TRANS, bool WALL>
+__global__ void __launch_bounds__(64, 6) k_band_solve_x(Geo g, XShape f, const double* __restrict__ fac,
+                                                        size_t fac_stride, double2* X,
+                                                        const double2* __restrict__ add, int helm, int zero_row0,
+                                                        double* __restrict__ pw, const double2* __restrict__ usub) {
     grid_dep_sync();
-    constexpr int NC1 = NL + (DIAG1 ? 1 : 0);
-    constexpr int NC2 = kB - NC1;
-    constexpr int NCM = NC1 > NC2 ? NC1 : NC2;
-    constexpr int MAXCH = MAXR / kRC;
-    static_assert(MAXR % kRC == 0, "whole chunks");
-    extern __shared__ __align__(16) unsigned char smem[];
-    double* Cb = reinterpret_cast<double*>(smem);  // [2][kRC][NCM][kSK]
+    __shared__ __align__(16) int2 stage_sh[2][2][kXR * 5 * kXK];
+    __shared__ __align__(16) int2 mid_sh[2][33 * kXK];
+    __shared__ int2 ex_sh[2][kXR][32], exu_sh[2][32];
+    const int nr = g.nr, nht = (g.nk + kXK - 1) / kXK;
     int bi = blockIdx.x;
-    const int kb = bi % g.ntile;
-    bi /= g.ntile;
-    const int im = bi % g.nm, v = bi / g.nm;
-    const int m = im - g.M;
-    const int mv = helm ? (v == 0 ? m + 1 : (v == 1 ? m - 1 : m)) : m;
-    const int k0 = kb * kSK;
-    const size_t S = (size_t)g.nr * g.nm * g.nk;
+    const int kb = bi % nht;
+    bi /= nht;
+    const int im = bi % g.nm, v = bi / g.nm, m = im - g.M;
+    const int mv = abs(helm ? (v == 0 ? m + 1 : (v == 1 ? m - 1 : m)) : m);
+    const int side = threadIdx.x >> 5, lane = threadIdx.x & 31, kk = lane >> 1, comp = lane & 1, k0 = kb * kXK;
+    const size_t S = (size_t)nr * g.nm * g.nk;
     const int slot = g.slot[blockIdx.y];
     const size_t off = (size_t)slot * g.fs;
-    fac += (size_t)slot * fac_stride;
-    X += off;
-    add = moved(add, off);
-    const double* T1 = fac + ((size_t)abs(mv) * g.ntile + kb) * (size_t)g.nr * kB * kSK;
-    const double* T2 = T1 + (size_t)g.nr * NC1 * kSK;
-    const int tid = threadIdx.x, sy = tid % kSK, comp = tid / kSK;
-    const int nr = g.nr, nch = (nr + kRC - 1) / kRC;
-    const bool on = k0 + sy < g.nk;
-    // this thread's column: the real or imaginary part of system (v, m, k0 + sy)
-    const double* xs = reinterpret_cast<const double*>(X + (size_t)v * S) + comp;
-    double x[MAXR];
-#pragma unroll
-    for (int j = 0; j < MAXR; ++j) x[j] = (on && j < nr) ? xs[2 * sidx(g, j, im, k0 + sy)] : 0.0;
-    // wall partials of the tentative velocity T^-1 x - usub (forward Helmholtz
-    // solves): the usub part now, the solution's part after the sweeps.
-    // v = 0, 1: d0 . (x/2) over rows 0..8 (d0 the wall row of D1 for u_r), minus
-    // d0 . usub_r on v = 0; the mean mode's u_z block: sum_j W_j (x - usub_z).
-    const bool mean_z = v == 2 && m == 0 && k0 + sy == 0;
+    const int2* T = reinterpret_cast<const int2*>(fac + (size_t)slot * fac_stride) + ((size_t)mv * nht + kb) * (size_t)f.tile;
+    const ptrdiff_t rs = (ptrdiff_t)g.nm * g.nk * 2;
+    XSide a;
+    a.side = side;
+    a.lane = lane;
+    a.n = f.chunks[side];
+    a.pad = side ? f.pad : 0;
+    a.on = k0 + kk < g.nk;
+    a.tin = T + f.in[side];
+    a.tout = T + f.out[side];
+    a.buf = stage_sh[side];
+    a.mid = mid_sh[side];
+    a.step = side ? -rs : rs;
+    const ptrdiff_t o0 = 2 * ((ptrdiff_t)v * S + (ptrdiff_t)im * g.nk + (a.on ? k0 + kk : k0)) + comp +
+                         (side ? (nr - 1 + a.pad) * rs : 0);
+    a.xp = reinterpret_cast<double*>(X + off) + o0;
+    a.ad = add ? reinterpret_cast<const double*>(add + off) + o0 : nullptr;
+    for (int i = lane; i < 33 * kXK / 2; i += 32) cp_async16(mid_sh[side] + 2 * i, T + f.mid[side] + 2 * i);
+    a.stage(0);
+    a.load(0);
+
+    // wall partials of the tentative velocity: the usub part, from memory,
+    // while the sweeps run (see the epilogue)
+    const double* us = WALL && usub ? reinterpret_cast<const double*>(usub + off) + comp : nullptr;
+    const double* d0 = g.D1 + (size_t)par_idx(m + 1) * nr * kB + 4;
     double wall_u = 0.0;
-    if (WALL && on && usub) {
-        const double* us = reinterpret_cast<const double*>(usub + off) + comp;
-        if (v == 0) {
-            const double* d0 = g.D1 + (size_t)par_idx(m + 1) * nr * kB + 4;
-#pragma unroll 1
-            for (int c = 0; c <= 8 && c < nr; ++c) wall_u = fma(__ldg(d0 + c), us[2 * sidx(g, c, im, k0 + sy)], wall_u);
-        } else if (mean_z) {
-#pragma unroll 1
-            for (int j = 0; j < nr; ++j) wall_u = fma(g.W[j], us[2 * (2 * S + sidx(g, j, im, 0))], wall_u);
-        }
+    if (WALL && us && a.on && v == 0 && side == 0) {
+        double t[9];
+#pragma unroll
+        for (int c = 0; c < 9; ++c) t[c] = us[2 * sidx(g, c, im, k0 + kk)];
+#pragma unroll
+        for (int c = 0; c < 9; ++c) wall_u = fma(__ldg(d0 + c), t[c], wall_u);
     }
-    auto stage = [&](int t) {  // chunk t of the sweep sequence into buffer t & 1
-        if (t >= 2 * nch) return;
-        const bool fwd = t < nch;
-        const int c = fwd ? t : 2 * nch - 1 - t;
-        const int rows = min(kRC, nr - c * kRC);
-        const int nc = fwd ? NC1 : NC2;
-        const double* src = (fwd ? T1 : T2) + (size_t)c * kRC * nc * kSK;
-        double* dst = Cb + (size_t)(t & 1) * kRC * NCM * kSK;
-        const int nseg = rows * nc * (kSK / 2);
-        for (int i = tid; i < nseg; i += 2 * kSK) cp_async16(dst + 2 * i, src + 2 * i);
-    };
-    stage(0);
-    cp_async_commit();
+    double(*x9)[32] = reinterpret_cast<double(*)[32]>(mid_sh[0]);  // rows 0..8 for the wall partials, after the middle
+    solve_fixed<TRANS, WALL>(a, T + f.wall + kk, helm ? g.shH[slot] : g.shP, helm, zero_row0, ex_sh, exu_sh, x9);
+    if (!WALL) return;
+    // wall partials, v = 0, 1: d0 . x / 2 over rows 0..8 (d0 the wall row of D1
+    // for u_r), minus d0 . usub_r on v = 0; the mean mode's u_z: sum_j W_j (x - usub_z)
+    double* P = pw + ((((size_t)slot * 3 + v) * g.nm + im) * g.nk + (k0 + kk)) * 2 + comp;
+    if (v < 2) {
+        if (side) return;
+        double acc = 0.0;
 #pragma unroll
-    for (int t = 0; t < MAXCH; ++t) {
-        if (t < nch) {
-            stage(t + 1);
-            cp_async_commit();
-            cp_async_wait1();
-            __syncthreads();
-            const double* C = Cb + (size_t)(t & 1) * kRC * NCM * kSK + sy;
-#pragma unroll
-            for (int r = 0; r < kRC; ++r) {
-                const int j = t * kRC + r;
-                if (j < nr) {
-                    double val = x[j];
-                    const bool full = !(NL == 8 && j > 8);
-#pragma unroll
-                    for (int e = 0; e < NL; ++e) {
-                        const int jj = j - NL + e;  // w1[e] of k_band_solve: oldest first
-                        if (jj >= 0 && (full || e >= NL - 4)) val = fma(-C[(r * NC1 + e) * kSK], x[jj >= 0 ? jj : 0], val);
-                    }
-                    if (DIAG1) val *= C[(r * NC1 + NL) * kSK];
-                    x[j] = val;
-                }
-            }
-            __syncthreads();
+        for (int c = 0; c < 9; ++c) acc = fma(__ldg(d0 + c), x9[c][lane], acc);
+        if (a.on) *P = fma(0.5, acc, -wall_u);
+    } else if (m == 0 && k0 == 0) {  // this block holds mode (0, 0): the lanes take the rows in turn, fixed order
+        __syncthreads();
+        if (side) return;
+        const double* xz = reinterpret_cast<const double*>(X + off) + comp;
+        double acc = 0.0;
+        for (int j = kk; j < nr; j += kXK) {
+            const size_t o = 2 * (2 * S + sidx(g, j, im, 0));
+            acc = fma(g.W[j], us ? xz[o] - us[o] : xz[o], acc);
         }
-    }
 #pragma unroll
-    for (int c = MAXCH - 1; c >= 0; --c) {
-        if (c < nch) {
-            const int t = 2 * nch - 1 - c;
-            stage(t + 1);
-            cp_async_commit();
-            cp_async_wait1();
-            __syncthreads();
-            const double* C = Cb + (size_t)(t & 1) * kRC * NCM * kSK + sy;
-            constexpr int O = DIAG1 ? 0 : 1;
-#pragma unroll
-            for (int r = kRC - 1; r >= 0; --r) {
-                const int j = c * kRC + r;
-                if (j < nr) {
-                    double val = x[j];
-                    const bool full = !(NU == 8 && j >= 4);
-#pragma unroll
-                    for (int e = NU - 1; e >= 0; --e) {
-                        const int jj = j + 1 + e;  // w2[e] of k_band_solve: nearest first (0 beyond nr)
-                        if (jj < MAXR && (full || e < 4)) val = fma(-C[(r * NC2 + O + e) * kSK], x[jj < MAXR ? jj : 0], val);
-                    }
-                    if (!DIAG1) val *= C[(r * NC2) * kSK];
-                    x[j] = val;
-                }
-            }
-            __syncthreads();
-        }
-    }
-    if (!on) return;
-    if (WALL) {
-        double* P = pw + ((((size_t)slot * 3 + v) * g.nm + im) * g.nk + (k0 + sy)) * 2 + comp;
-        if (v < 2) {
-            const double* d0 = g.D1 + (size_t)par_idx(m + 1) * nr * kB + 4;
-            double acc = 0.0;
-#pragma unroll
-            for (int c = 0; c <= 8; ++c)
-                if (c < nr) acc = fma(__ldg(d0 + c), 0.5 * x[c], acc);
-            *P = acc - wall_u;
-        } else if (mean_z) {
-            double acc = 0.0;
-#pragma unroll
-            for (int j = 0; j < MAXR; ++j)
-                if (j < nr) acc = fma(g.W[j], x[j], acc);
-            *P = acc - wall_u;
-        }
-    }
-    double* xo = reinterpret_cast<double*>(X + (size_t)v * S) + comp;
-    const double* ad = add ? reinterpret_cast<const double*>(add + (size_t)v * S) + comp : nullptr;
-#pragma unroll
-    for (int j = 0; j < MAXR; ++j) {
-        if (j < nr) {
-            const size_t o = 2 * sidx(g, j, im, k0 + sy);
-            double val = (zero_row0 && j == 0) ? 0.0 : x[j];
-            if (ad) val += ad[o];
-            xo[o] = val;
-        }
+        for (int d = 2; d < 32; d <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
+        if (kk == 0) *P = acc;
     }
 }
 
@@ -1816,36 +2104,49 @@ void launch_baseT(const Geo& g, const double2* nb, double2* ub, cudaStream_t s) 
 
 // trans selects the transposed coefficient layout; zero_row0 writes 0 to the
 // wall row of the solution; pw (forward Helmholtz solves only) receives the
-// wall partials of the tentative velocity, with usub subtracted
+// wall partials of the tentative velocity, with usub subtracted.  The slots
+// whose table is in fixed point go to the integer kernel, the others to the
+// FP64 one (a context's tables are of one kind but for its physics).
 static void launch_band_solve(const Geo& g, const double* fac, size_t fac_stride, double2* X, const double2* add,
                               int helm, int trans, int zero_row0, cudaStream_t s, double* pw = nullptr,
                               const double2* usub = nullptr) {
-    const dim3 nblocks((unsigned)((helm ? 3 : 1) * g.nm * g.ntile), (unsigned)g.nb);
-    // columns in registers for the Helmholtz solves (three systems per mode:
-    // several warps per scheduler hide the dependent chain); the pressure
-    // solve, one system per mode and about one warp per scheduler, keeps the
-    // shared-memory form, which measured faster there.  Only the forward
-    // Helmholtz instance carries the wall-partial epilogue (pw).
-    if (helm && g.nr <= kRegRows) {
-        const size_t sm = 2 * (size_t)kRC * 9 * kSK * sizeof(double);
-        auto go = [&](auto kernel, double* wall_pw, const double2* wall_u) {
-            smem_limit((const void*)kernel);
-            launch_serial(kernel, nblocks, 2 * kSK, sm, s, g, fac, fac_stride, X, add, helm, zero_row0, wall_pw,
-                          wall_u);
-        };
-        if (!trans && pw) go(k_band_solve_reg<4, 8, false, kRegRows, true>, pw, usub);
-        else if (!trans) go(k_band_solve_reg<4, 8, false, kRegRows, false>, nullptr, nullptr);
-        else go(k_band_solve_reg<8, 4, true, kRegRows, false>, nullptr, nullptr);
-        return;
+    const FxShape fx = fx_shape(g.nr);
+    Geo gx = g, gd = g;
+    gx.nb = gd.nb = 0;
+    for (int b = 0; b < g.nb; ++b) {
+        Geo& to = (helm ? g.fxH[g.slot[b]] : g.fxP) && std::max(fx.chunks[0], fx.chunks[1]) <= kXChunks ? gx : gd;
+        to.slot[to.nb++] = g.slot[b];
     }
-    const size_t sm = (size_t)g.nr * kSK * sizeof(double2) + 2 * (size_t)kRC * 9 * kSK * sizeof(double);
-    auto go = [&](auto kernel, double* wall_pw, const double2* wall_u) {
-        smem_limit((const void*)kernel);
-        launch_serial(kernel, nblocks, 2 * kSK, sm, s, g, fac, fac_stride, X, add, helm, zero_row0, wall_pw, wall_u);
-    };
-    if (!trans && pw) go(k_band_solve<4, 8, false, true>, pw, usub);
-    else if (!trans) go(k_band_solve<4, 8, false, false>, nullptr, nullptr);
-    else go(k_band_solve<8, 4, true, false>, nullptr, nullptr);
+    if (gx.nb) {
+        XShape xs{};
+        xs.pad = fx.pad;
+        xs.wall = (int)fx.wall;
+        xs.tile = (int)fx.tile;
+        for (int i = 0; i < 2; ++i) {
+            xs.chunks[i] = fx.chunks[i];
+            xs.in[i] = (int)fx.in[i];
+            xs.out[i] = (int)fx.out[i];
+            xs.mid[i] = (int)fx.mid[i];
+        }
+        auto go = [&](auto kernel) {
+            const dim3 grid((unsigned)((helm ? 3 : 1) * g.nm * ((g.nk + kXK - 1) / kXK)), (unsigned)gx.nb);
+            launch_serial(kernel, grid, 64, 0, s, gx, xs, fac, fac_stride, X, add, helm, zero_row0, pw, usub);
+        };
+        if (!trans && pw) go(k_band_solve_x<false, true>);
+        else if (!trans) go(k_band_solve_x<false, false>);
+        else go(k_band_solve_x<true, false>);
+    }
+    if (gd.nb) {
+        const size_t sm = (size_t)g.nr * kSK * sizeof(double2) + 2 * (size_t)kRC * 9 * kSK * sizeof(double);
+        auto go = [&](auto kernel) {
+            smem_limit((const void*)kernel);
+            const dim3 grid((unsigned)((helm ? 3 : 1) * g.nm * g.ntile), (unsigned)gd.nb);
+            launch_serial(kernel, grid, 2 * kSK, sm, s, gd, fac, fac_stride, X, add, helm, zero_row0, pw, usub);
+        };
+        if (!trans && pw) go(k_band_solve<4, 8, false, true>);
+        else if (!trans) go(k_band_solve<4, 8, false, false>);
+        else go(k_band_solve<8, 4, true, false>);
+    }
 }
 
 void launch_stage_div(const Geo& g, const double2* F, double2* q, cudaStream_t s) {

@@ -22,10 +22,17 @@ struct Geo {
     const double* D1;    // [2][nr][13]
     const double* Lb;    // [M+2][nr][13]  L_m / (2 Re), no k_z^2 (that sits in dgt)
     int ntile;           // k tiles of kSK values in the factor tables
-    const double* facH;  // M+2 Helmholtz matrices, A x = b rows, tiled (4 forward | 9 backward columns)
-    const double* facP;  // M+1 pressure matrices, same layout
-    const double* facHT; // transposed-solve rows, tiled (9 forward | 4 backward columns)
+    // banded factors, direct and transposed: FP64 rows (4 forward | 9 backward,
+    // 9 | 4 columns, tiled) or fixed-point tables (setup.hpp), see fxH and fxP
+    const double* facH;  // M+2 Helmholtz matrices
+    const double* facP;  // M+1 pressure matrices
+    const double* facHT;
     const double* facPT;
+    // 1: the slot's Helmholtz tables (fxP: the pressure tables) are in fixed
+    // point, with the multipliers of column 0 of L scaled by 2^-shH (2^-shP)
+    unsigned char fxH[kMaxBatch];
+    int shH[kMaxBatch];
+    int fxP, shP;
     const double* infl;  // [nm][3][nr][nk] (k fastest)
     const double* fluxg; // [nr]
     const double2* Uh;   // [nr]

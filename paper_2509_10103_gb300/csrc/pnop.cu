@@ -248,9 +248,11 @@ template <class T2> std::vector<T2> twiddle_table(int N) {
 // on first use; the grid-only tables (pressure factors) are written once.
 void upload_slot_operators(pnop_ctx* c, int slot, const pnop::HostOps& h) {
     const size_t ns = (size_t)c->nslot;
-    auto put = [&](double*& dst, const std::vector<double>& v, size_t slots, size_t at) {
-        if (!dst) dst = (double*)c->dalloc(std::max<size_t>(1, v.size()) * slots * sizeof(double));
-        ck(cudaMemcpy(dst + at * v.size(), v.data(), v.size() * sizeof(double), cudaMemcpyHostToDevice), "upload");
+    // v into the table of slot `at` (stride `stride` values, at least v.size())
+    auto put = [&](double*& dst, const std::vector<double>& v, size_t slots, size_t at, size_t stride = 0) {
+        stride = std::max(stride, v.size());
+        if (!dst) dst = (double*)c->dalloc(std::max<size_t>(1, stride) * slots * sizeof(double));
+        ck(cudaMemcpy(dst + at * stride, v.data(), v.size() * sizeof(double), cudaMemcpyHostToDevice), "upload");
     };
     {
         // device bands hold L_m / (2 Re): the explicit Crank-Nicolson half B = 1/dt + L/(2 Re)
@@ -268,12 +270,20 @@ void upload_slot_operators(pnop_ctx* c, int slot, const pnop::HostOps& h) {
         put(c->d_dgt, dg, ns, slot);
         c->geo.sNk = dg.size();
     }
-    put(c->d_facH, h.facH, ns, slot);
-    put(c->d_facHT, h.facHT, ns, slot);
-    c->geo.sFacH = h.facH.size();
+    // banded factors: a slot's table has room for either form
+    const size_t nht = (h.d.nk + pnop::kTileX - 1) / pnop::kTileX, tile = nht * pnop::fx_shape(h.d.nr).tile;
+    const size_t fp64 = (size_t)h.ntile * h.d.nr * pnop::kBand * pnop::kTileK;
+    const size_t strideH = (h.d.M + 2) * std::max(fp64, tile), strideP = (h.d.M + 1) * std::max(fp64, tile);
+    put(c->d_facH, h.fxH.ok ? h.fxH.direct : h.facH, ns, slot, strideH);
+    put(c->d_facHT, h.fxH.ok ? h.fxH.transposed : h.facHT, ns, slot, strideH);
+    c->geo.sFacH = strideH;
+    c->geo.fxH[slot] = h.fxH.ok;
+    c->geo.shH[slot] = h.fxH.shift;
     if (!c->d_facP) {
-        put(c->d_facP, h.facP, 1, 0);
-        put(c->d_facPT, h.facPT, 1, 0);
+        put(c->d_facP, h.fxP.ok ? h.fxP.direct : h.facP, 1, 0, strideP);
+        put(c->d_facPT, h.fxP.ok ? h.fxP.transposed : h.facPT, 1, 0, strideP);
+        c->geo.fxP = h.fxP.ok;
+        c->geo.shP = h.fxP.shift;
     }
     put(c->d_infl, h.infl, ns, slot);
     c->geo.sInfl = h.infl.size();
@@ -1384,8 +1394,7 @@ pnop::HostOps batch_prepare(const pnop_ctx* c, const pnop_params* p) {
     hs.W = c->h.W;
     hs.D1 = c->h.D1;
     hs.D2 = c->h.D2;
-    hs.facP = c->h.facP;
-    hs.facPT = c->h.facPT;
+    hs.phi = c->h.phi;
     hs.ph = {p->Re, p->Wo, p->A, p->dt, p->tau0};
     std::string err;
     if (!pnop::build_operators(hs, err, true)) throw Status(PNOP_ERR_UNSUPPORTED, err);

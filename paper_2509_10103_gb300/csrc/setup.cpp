@@ -10,6 +10,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
+#include <cstring>
 #include <random>
 #include <thread>
 #include <vector>
@@ -281,13 +282,6 @@ static void scatter_factors(std::vector<double>& dst, int mat, int k, int nr, in
         for (int e = 0; e < kBand; ++e) dst[fac_index(mat, k, j, e, nr, ntile, nc1)] = f[(size_t)j * kBand + e];
 }
 
-static void gather_factors(const std::vector<double>& src, int mat, int k, int nr, int ntile, int nc1,
-                           std::vector<double>& f) {
-    f.resize((size_t)nr * kBand);
-    for (int j = 0; j < nr; ++j)
-        for (int e = 0; e < kBand; ++e) f[(size_t)j * kBand + e] = src[fac_index(mat, k, j, e, nr, ntile, nc1)];
-}
-
 // Row-local coefficients of A^T = U^T L^T from the factors of A: row j holds
 // U_{j-8+e, j} (e = 0..7, oldest first), 1/U_jj, L_{j+1+e, j} (e = 0..3).
 static std::vector<double> transpose_factors(int nr, const std::vector<double>& f) {
@@ -304,6 +298,281 @@ static std::vector<double> transpose_factors(int nr, const std::vector<double>& 
         }
     }
     return t;
+}
+
+// value in fixed point, as the two signed digits the device reads (low, high)
+static double fx_bits(long long c) {
+    if ((unsigned)(c & 0xFFFFFFFFll) == 0x80000000u) ++c;  // keeps the low digit above -2^31 (x_dot4's sums)
+    const int lo = (int)(unsigned)(c & 0xFFFFFFFFll);
+    const unsigned hi = (unsigned)(int)((c - lo) >> 32);
+    const unsigned long long b = ((unsigned long long)hi << 32) | (unsigned)lo;
+    double d;
+    std::memcpy(&d, &b, sizeof d);
+    return d;
+}
+// -a b in fixed point (the product's rounding error included)
+static long long fx_neg(double a, double b) {
+    constexpr double s = (double)(1ll << kFxBits);
+    const double p = a * b, e = std::fma(a, b, -p);
+    return -(std::llround(p * s) + std::llround(e * s));
+}
+
+// The two-sided factorisation of one matrix (layout notes in setup.hpp), by
+// positions: l[s][p][e] = N(p, p-4+e) for the outer columns, u[s][p][e] =
+// U(p, p+1+e), d[s][p] = 1/D, all of side s, and the inverse of the middle block.
+struct Twist {
+    std::vector<double> l[2], u[2], d[2];
+    double mid[8][8];  // S^-1 by rows h-4..h+3
+};
+// G = S^-1: Gauss-Jordan with partial pivoting, then one Newton step
+// G += G (I - S G) with the residual's products and sums compensated.
+static bool invert8(const double (&S)[8][8], double (&G)[8][8]) {
+    double a[8][16];
+    for (int i = 0; i < 8; ++i)
+        for (int j = 0; j < 8; ++j) {
+            a[i][j] = S[i][j];
+            a[i][8 + j] = i == j;
+        }
+    for (int c = 0; c < 8; ++c) {
+        int p = c;
+        for (int i = c + 1; i < 8; ++i)
+            if (std::fabs(a[i][c]) > std::fabs(a[p][c])) p = i;
+        if (a[p][c] == 0.0 || !std::isfinite(a[p][c])) return false;
+        if (p != c) std::swap(a[p], a[c]);
+        const double inv = 1.0 / a[c][c];
+        for (int j = c; j < 16; ++j) a[c][j] *= inv;
+        for (int i = 0; i < 8; ++i) {
+            const double m = a[i][c];
+            if (i == c || m == 0.0) continue;
+            for (int j = c; j < 16; ++j) a[i][j] = std::fma(-m, a[c][j], a[i][j]);
+        }
+    }
+    double R[8][8];
+    for (int i = 0; i < 8; ++i)
+        for (int j = 0; j < 8; ++j) {
+            double s = i == j, e = 0.0;
+            for (int k = 0; k < 8; ++k) {
+                const double p = -S[i][k] * a[k][8 + j], pe = std::fma(-S[i][k], a[k][8 + j], -p), t = s + p, z = t - s;
+                e += ((s - (t - z)) + (p - z)) + pe;
+                s = t;
+            }
+            R[i][j] = s + e;
+        }
+    for (int i = 0; i < 8; ++i)
+        for (int j = 0; j < 8; ++j) {
+            double d = 0.0;
+            for (int k = 0; k < 8; ++k) d = std::fma(a[i][8 + k], R[k][j], d);
+            G[i][j] = a[i][8 + j] + d;
+        }
+    return true;
+}
+static bool twist_factor(const Band& A, const FxShape& f, Twist& t) {
+    const int n = A.n, h = f.h, B = 8, W = 2 * B + 1;
+    thread_local std::vector<double> w;
+    w.assign((size_t)n * W, 0.0);
+    auto at = [&](int i, int j) -> double& { return w[(size_t)i * W + (j - i + B)]; };
+    for (int i = 0; i < n; ++i)
+        for (int j = std::max(0, i - kLo); j <= std::min(n - 1, i + kUp); ++j) at(i, j) = A.get(i, j);
+    for (int s = 0; s < 2; ++s) {
+        const int np = 4 * f.chunks[s], pad = s ? f.pad : 0;
+        t.l[s].assign((size_t)np * 4, 0.0);
+        t.u[s].assign((size_t)np * 8, 0.0);
+        t.d[s].assign(np, 0.0);
+        auto row = [&](int p) { return s ? n - 1 - (p - pad) : p; };
+        for (int p = pad; p < np - 4; ++p) {
+            const int i = row(p);
+            const double piv = at(i, i);
+            if (piv == 0.0 || !std::isfinite(piv)) return false;
+            t.d[s][p] = 1.0 / piv;
+            for (int e = 0; e < 8; ++e) {
+                const int q = p + 1 + e, j = row(q);
+                if (j < 0 || j >= n) break;
+                const double v = at(i, j);
+                if (v != 0.0 && e >= 4 && (s || p > 3 || q > 8)) return false;
+                t.u[s][(size_t)p * 8 + e] = v * t.d[s][p];
+            }
+            for (int q = p + 1; q <= p + 4; ++q) {
+                const int j = row(q);
+                const double m = at(j, i) / piv;
+                t.l[s][(size_t)q * 4 + (p - q + 4)] = m;
+                if (m == 0.0) continue;
+                for (int c = 1; c <= 8; ++c) {
+                    const int k = row(p + c);
+                    if (k < 0 || k >= n || std::abs(k - j) > B) break;
+                    at(j, k) -= m * at(i, k);
+                }
+            }
+        }
+    }
+    double S[8][8];
+    for (int i = 0; i < 8; ++i)
+        for (int j = 0; j < 8; ++j) S[i][j] = at(h - 4 + i, h - 4 + j);
+    return invert8(S, t.mid);
+}
+// positions of a side's half of the middle as rows of the block: own, then the other side's
+static int mid_row(int s, int i) { return i < 4 ? (s ? 7 - i : i) : (s ? i - 4 : 11 - i); }
+
+// Residual of the two-sided solve of one random system, relative as in
+// band_backward_error.
+static double twist_backward_error(const Band& A, const FxShape& f, const Twist& t, unsigned seed) {
+    const int n = A.n;
+    std::mt19937_64 g(seed);
+    std::uniform_real_distribution<double> U(-1, 1);
+    std::vector<double> b(n), x(n);
+    for (double& v : b) v = U(g);
+    double mid[8];
+    std::vector<double> y[2];
+    for (int s = 0; s < 2; ++s) {
+        const int np = 4 * f.chunks[s], pad = s ? f.pad : 0;
+        y[s].assign(np, 0.0);
+        for (int p = pad; p < np; ++p) {
+            double v = b[s ? n - 1 - (p - pad) : p];
+            for (int e = 0; e < 4; ++e)
+                if (p - 4 + e >= 0) v -= t.l[s][(size_t)p * 4 + e] * y[s][p - 4 + e];
+            y[s][p] = v;
+        }
+        for (int i = 0; i < 4; ++i) mid[mid_row(s, i)] = y[s][np - 4 + i];
+    }
+    for (int s = 0; s < 2; ++s) {
+        const int np = 4 * f.chunks[s], pad = s ? f.pad : 0;
+        std::vector<double> xs(np + 8, 0.0);
+        for (int i = 0; i < 4; ++i) {
+            double v = 0;
+            for (int c = 0; c < 8; ++c) v += t.mid[mid_row(s, i)][c] * mid[c];
+            xs[np - 4 + i] = v;
+        }
+        for (int p = np - 5; p >= pad; --p) {
+            double v = y[s][p] * t.d[s][p];
+            for (int e = 0; e < 8; ++e) v -= t.u[s][(size_t)p * 8 + e] * xs[p + 1 + e];
+            xs[p] = v;
+        }
+        for (int p = pad; p < np; ++p) x[s ? n - 1 - (p - pad) : p] = xs[p];
+    }
+    double rmax = 0, amax = 0, xmax = 0;
+    for (int j = 0; j < n; ++j) {
+        double r = -b[j], arow = 0;
+        for (int c = std::max(0, j - kLo); c <= std::min(n - 1, j + kUp); ++c) {
+            r += A.get(j, c) * x[c];
+            arow += std::fabs(A.get(j, c));
+        }
+        rmax = std::max(rmax, std::fabs(r));
+        amax = std::max(amax, arow);
+        xmax = std::max(xmax, std::fabs(x[j]));
+    }
+    const double e = rmax / (amax * xmax + 1e-300);
+    return std::isfinite(e) ? e : 1.0;
+}
+
+// Largest row sum of the multipliers of one factorisation (column 0 apart,
+// which is scaled to at most 1), and the largest entry of that column.
+static void fx_measure(const FxShape& f, const Twist& t, double& sum, double& col0) {
+    for (int s = 0; s < 2; ++s) {
+        const int np = 4 * f.chunks[s];
+        for (int p = 0; p < np; ++p) {
+            double l = 0, u = 0, lt = 0, ut = 0;  // rows and columns of N and U
+            for (int e = 0; e < 4; ++e) {
+                const double a = std::fabs(t.l[s][(size_t)p * 4 + e]);
+                const bool first = s == 0 && p - 4 + e == 0;
+                if (first) col0 = std::max(col0, a);
+                l += first ? std::min(a, 1.0) : a;
+                if (p + 1 + e < np) {
+                    const double b = std::fabs(t.l[s][(size_t)(p + 1 + e) * 4 + 3 - e]);
+                    lt += s == 0 && p == 0 ? std::min(b, 1.0) : b;
+                }
+            }
+            for (int e = 0; e < 8; ++e) {
+                u += std::fabs(t.u[s][(size_t)p * 8 + e]);
+                if (p - 1 - e >= 0) ut += std::fabs(t.u[s][(size_t)(p - 1 - e) * 8 + e]);
+            }
+            const double worst = std::max(std::max(l, u), std::max(lt, ut));
+            if (!(worst <= sum)) sum = worst;  // NaN included
+        }
+    }
+}
+
+// Writes a factorisation into the tables at (mat, k).  False when 1/D or S^-1 is
+// outside the range of its format.
+static bool fx_write(FixedTable& tab, int mat, int k, int nht, const FxShape& f, const Twist& t) {
+    const size_t base = ((size_t)mat * nht + k / kTileX) * f.tile, kk = k % kTileX;
+    auto mult = [&](double v, double scale) { return fx_bits(fx_neg(v, scale)); };
+    auto pair = [&](size_t row, int e) { return ((row * 2 + e / 2) * kTileX + kk) * 2 + e % 2; };
+    for (int s = 0; s < 2; ++s) {
+        const int np = 4 * f.chunks[s];
+        auto L = [&](int p, int q) {  // N(p, q), q < p
+            const bool first = s == 0 && q == 0;
+            return q < 0 || p >= np ? 0.0 : mult(t.l[s][(size_t)p * 4 + (q - p + 4)], first ? std::ldexp(1.0, -tab.shift) : 1.0);
+        };
+        auto U = [&](int p, int q) { return p < 0 || q >= np ? 0.0 : mult(t.u[s][(size_t)p * 8 + (q - p - 1)], 1.0); };
+        for (int p = 0; p < np; ++p) {
+            const size_t in = base + f.in[s], out = base + f.out[s] + (size_t)(p / 4) * 20 * kTileX;
+            for (int e = 0; e < 4; ++e) {
+                // the middle rows couple inwards through S alone
+                const int q = p - 4 + e;
+                const bool inner = q >= np - 4;
+                tab.direct[in + pair(p, e)] = inner ? 0.0 : L(p, q);
+                tab.transposed[in + pair(p, e)] = inner ? 0.0 : U(q, p);
+                if (p < np - 4) {
+                    tab.direct[out + pair(p % 4, e)] = U(p, p + 1 + e);
+                    tab.transposed[out + pair(p % 4, e)] = L(p + 1 + e, p);
+                }
+            }
+        }
+        // 1/D = D' 2^(q - 60), D' of at most 62 bits with q + 128 as its low byte
+        // (the bits above are rounded for the byte to be part of the value).  The
+        // rows of a chunk of four share q except in the first chunk (the wall row).
+        // A row whose 1/D is more than 2^6 below the largest of its chunk would
+        // keep too few bits.
+        for (int p = 0; p < np - 4;) {
+            const int end = p < 4 ? p + 1 : p + 4;
+            int lo = 1 << 20, hi = -(1 << 20);
+            for (int i = p; i < end; ++i) {
+                int q = 0;
+                std::frexp(t.d[s][i], &q);
+                if (t.d[s][i] == 0.0) continue;  // empty position
+                lo = std::min(lo, q);
+                hi = std::max(hi, q);
+            }
+            if (lo > hi) lo = hi = 0;
+            const int q = hi - 2;
+            if (hi - lo > 6 || q < -127 || q > 127) return false;
+            for (; p < end; ++p) {
+                const long long scaled = std::llround(std::ldexp(t.d[s][p], 60 - q)), byte = q + 128;
+                const size_t o = base + f.out[s] + (size_t)(p / 4) * 20 * kTileX + (16 + p % 4) * kTileX + kk;
+                tab.direct[o] = tab.transposed[o] = fx_bits(((scaled - byte + 128) >> 8) * 256 + byte);
+            }
+        }
+        // S^-1 scaled by a power of two to row sums of at most 1
+        for (int tr = 0; tr < 2; ++tr) {
+            auto& dst = tr ? tab.transposed : tab.direct;
+            double sum = 0;
+            for (int i = 0; i < 4; ++i) {
+                double r = 0;
+                for (int c = 0; c < 8; ++c) r += std::fabs(tr ? t.mid[c][mid_row(s, i)] : t.mid[mid_row(s, i)][c]);
+                if (!(r <= sum)) sum = r;
+            }
+            int q = 0;
+            if (!std::isfinite(sum) || sum == 0.0) return false;
+            std::frexp(sum, &q);
+            if (q < -900 || q > 900) return false;
+            const size_t o = base + f.mid[s];
+            for (int i = 0; i < 4; ++i)
+                for (int c = 0; c < 8; ++c) {
+                    const int a = mid_row(s, i), b = mid_row(s, c);
+                    const double v = tr ? t.mid[b][a] : t.mid[a][b];
+                    dst[o + ((size_t)(i * 4 + c / 2) * kTileX + kk) * 2 + c % 2] =
+                        fx_bits(std::llround(std::ldexp(v, kFxBits - q)));
+                }
+            dst[o + 32 * kTileX + kk] = fx_bits(q);
+        }
+    }
+    for (int i = 0; i < 4; ++i)
+        for (int e = 0; e < 4; ++e) {  // U(i, 5 + e), the part beyond four columns
+            const int c = 5 + e;
+            const double v = c - i > 4 ? mult(t.u[0][(size_t)i * 8 + (c - i - 1)], 1.0) : 0.0;
+            tab.direct[base + f.wall + (size_t)(i * 4 + e) * kTileX + kk] = v;
+            tab.transposed[base + f.wall + (size_t)(e * 4 + i) * kTileX + kk] = v;
+        }
+    return true;
 }
 
 static Band laplacian_band(const HostOps& h, int mabs, double kz) {
@@ -334,7 +603,7 @@ static Band pressure_band(const HostOps& h, int mabs, double kz) {
     return A;
 }
 
-// fn(k) for k = 0..n-1 on up to 16 host threads; fn touches only data of its own k.
+// fn(i, thread) for i = 0..n-1 on up to 16 host threads; fn touches only data of its own i.
 template <class F> static void parallel_k(int n, F&& fn) {
     const int T = std::max(1, std::min<int>({n, 16, (int)std::max(1u, std::thread::hardware_concurrency())}));
     if (T == 1) {
@@ -347,6 +616,87 @@ template <class F> static void parallel_k(int n, F&& fn) {
             for (int k = t; k < n; k += T) fn(k, t);
         });
     for (auto& x : th) x.join();
+}
+
+// Factors nmat matrices per k: calls each(ma, k, f) with the LU factors (FP64,
+// without pivoting; worst: its largest backward error) and fills the device
+// tables, in fixed point where every row of every matrix fits and the two-sided
+// elimination is as stable as the LU has to be, else in FP64.  Work is split by
+// (matrix, table tile), so that a host thread writes whole tiles.  False when a
+// LU breaks down.
+template <class F, class E>
+static bool factor_tables(const HostOps& h, FixedTable& t, std::vector<double>& fac, std::vector<double>& facT,
+                          int nmat, F&& matrix, E&& each, double& worst) {
+    const int nr = h.d.nr, nk = h.d.nk, nht = (nk + kTileX - 1) / kTileX;
+    const FxShape shape = fx_shape(nr);
+    auto kz = [&](int k) { return 2.0 * M_PI * k / h.d.Lz; };
+    t.ok = nr >= kFxMinRows;
+    t.shift = 0;
+    fac.clear();
+    facT.clear();
+    t.direct.clear();
+    t.transposed.clear();
+    if (t.ok) {
+        // column 0 of N is column 0 of A over the wall row's diagonal: the
+        // wall-side rows of A off its diagonal depend on neither m (but for its
+        // parity, which does not reach them) nor k
+        const Band A = matrix(std::min(1, nmat - 1), kz(0));
+        double col = 0;
+        for (int j = 1; j <= kLo; ++j) col = std::max(col, std::fabs(A.get(j, 0) / A.get(0, 0)));
+        if (std::isfinite(col))
+            while (std::ldexp(col, -t.shift) > 1.0) ++t.shift;
+        t.direct.assign((size_t)nmat * nht * shape.tile, 0.0);
+        t.transposed.assign(t.direct.size(), 0.0);
+    }
+    std::vector<double> err_t(16, 0.0), sum(16, 0.0), col(16, 0.0);
+    std::vector<int> fail(16, 0), unfit(16, 0);
+    parallel_k(nmat * nht, [&](int item, int th) {
+        const int ma = item / nht, k0 = item % nht * kTileX;
+        std::vector<double> f;
+        Twist w;
+        double growth = 0;
+        for (int k = k0; k < std::min(nk, k0 + kTileX) && !fail[th]; ++k) {
+            const Band A = matrix(ma, kz(k));
+            if (!band_lu(A, f, growth)) {
+                fail[th] = 1;
+                return;
+            }
+            err_t[th] = std::max(err_t[th], band_backward_error(A, f, 1234u + ma * 977u + k));
+            each(ma, k, f);
+            if (!t.ok || unfit[th]) continue;
+            if (!twist_factor(A, shape, w) || !(twist_backward_error(A, shape, w, 99u + ma * 977u + k) < 1e-12)) {
+                unfit[th] = 1;
+                continue;
+            }
+            fx_measure(shape, w, sum[th], col[th]);
+            if (!(sum[th] <= kFxRowSum) || !(std::ldexp(col[th], -t.shift) <= 1.0) ||
+                !fx_write(t, ma, k, nht, shape, w))
+                unfit[th] = 1;
+        }
+    });
+    bool ok = t.ok;
+    for (int th = 0; th < 16; ++th) {
+        if (fail[th]) return false;
+        ok = ok && !unfit[th];
+        worst = std::max(worst, err_t[th]);
+    }
+    t.ok = ok;
+    if (ok) return true;
+    t = FixedTable{};
+    const int nt = h.ntile;
+    fac.assign((size_t)nmat * nt * nr * kBand * kTileK, 0.0);
+    facT.assign(fac.size(), 0.0);
+    parallel_k(nmat * nt, [&](int item, int) {
+        const int ma = item / nt, k0 = item % nt * kTileK;
+        std::vector<double> f;
+        double growth = 0;
+        for (int k = k0; k < std::min(nk, k0 + kTileK); ++k) {
+            band_lu(matrix(ma, kz(k)), f, growth);
+            scatter_factors(fac, ma, k, nr, nt, kNc1Direct, f);
+            scatter_factors(facT, ma, k, nr, nt, kNc1Transposed, transpose_factors(nr, f));
+        }
+    });
+    return true;
 }
 
 bool build_operators(HostOps& h, std::string& err, bool reuse_pressure) {
@@ -369,124 +719,105 @@ bool build_operators(HostOps& h, std::string& err, bool reuse_pressure) {
             h.Lb[((size_t)ma * nr + j) * kBand + kLo] -= (double)ma * ma * h.invr[j] * h.invr[j];
         }
     }
-    const int nt = h.ntile = (nk + kTileK - 1) / kTileK;
-    const int D = kNc1Direct, T = kNc1Transposed;
-    const size_t pressure_size = (size_t)(M + 1) * nt * nr * kBand * kTileK;
-    // the pressure factors depend on the grid only: a caller that built them
-    // for this grid before may keep them
-    const bool pressure = !(reuse_pressure && h.facP.size() == pressure_size && h.facPT.size() == pressure_size);
-    h.facH.assign((size_t)(M + 2) * nt * nr * kBand * kTileK, 0.0);
-    h.facHT.assign(h.facH.size(), 0.0);
-    if (pressure) {
-        h.facP.assign(pressure_size, 0.0);
-        h.facPT.assign(pressure_size, 0.0);
-    }
-    // every k owns its own factor entries, so the k loop runs on host threads
-    std::vector<double> worst_t(16, 0.0);
-    std::vector<int> fail_t(16, 0);
-    parallel_k(nk, [&](int k, int t) {
-        std::vector<double> f;
-        double growth = 0;
-        const double kz = 2.0 * M_PI * k / d.Lz;
-        for (int ma = 0; ma <= M + 1; ++ma) {
-            Band A = helmholtz_band(h, ma, kz);
-            if (!band_lu(A, f, growth)) {
-                fail_t[t] = 1;
-                return;
-            }
-            worst_t[t] = std::max(worst_t[t], band_backward_error(A, f, 1234u + ma * 977u + k));
-            scatter_factors(h.facH, ma, k, nr, nt, D, f);
-            scatter_factors(h.facHT, ma, k, nr, nt, T, transpose_factors(nr, f));
-        }
-        if (!pressure) return;
-        for (int ma = 0; ma <= M; ++ma) {
-            if (ma == 0 && k == 0) {
-                // singular Neumann problem of the mean mode: never used (p = 0)
-                std::vector<double> id((size_t)nr * kBand, 0.0);
-                for (int j = 0; j < nr; ++j) id[(size_t)j * kBand + kLo] = 1.0;
-                scatter_factors(h.facP, ma, k, nr, nt, D, id);
-                scatter_factors(h.facPT, ma, k, nr, nt, T, transpose_factors(nr, id));
-                continue;
-            }
-            Band A = pressure_band(h, ma, kz);
-            if (!band_lu(A, f, growth)) {
-                fail_t[t] = 2;
-                return;
-            }
-            worst_t[t] = std::max(worst_t[t], band_backward_error(A, f, 4321u + ma * 131u + k));
-            scatter_factors(h.facP, ma, k, nr, nt, D, f);
-            scatter_factors(h.facPT, ma, k, nr, nt, T, transpose_factors(nr, f));
-        }
-    });
+    h.ntile = (nk + kTileK - 1) / kTileK;
     double worst = 0;
-    for (int t = 0; t < 16; ++t) {
-        if (fail_t[t]) {
-            err = fail_t[t] == 1 ? "Helmholtz band LU failed" : "pressure band LU failed";
+    // Pressure factors, and the pressure phi of a unit wall datum for every
+    // (|m|, k): they depend on the grid only, a caller that built them for this
+    // grid before may keep them.
+    const size_t sys = (size_t)(M + 1) * nk * nr;
+    auto at = [&](int ma, int k) { return ((size_t)ma * nk + k) * nr; };
+    if (!(reuse_pressure && h.phi.size() == sys)) {
+        h.phi.assign(sys, 0.0);
+        const bool done = factor_tables(
+            h, h.fxP, h.facP, h.facPT, M + 1,
+            [&](int ma, double kz) {
+                if (ma || kz != 0.0) return pressure_band(h, ma, kz);
+                Band I{nr, std::vector<double>((size_t)nr * kBand, 0.0)};  // singular mean mode: never used (p = 0)
+                for (int j = 0; j < nr; ++j) I.at(j, j) = 1.0;
+                return I;
+            },
+            [&](int ma, int k, const std::vector<double>& f) {
+                if (ma == 0 && k == 0) return;
+                std::vector<double> x(nr, 0.0);
+                x[0] = 1.0;
+                band_solve(nr, f, x);
+                std::copy(x.begin(), x.end(), h.phi.begin() + at(ma, k));
+            },
+            worst);
+        if (!done) {
+            err = "pressure band LU failed";
             return false;
         }
-        worst = std::max(worst, worst_t[t]);
     }
-    std::vector<double> f, fac_tmp;
-    double growth = 0;
+    // Helmholtz factors, and the Helmholtz responses to -grad(phi) with u = 0 at
+    // the wall: u+ and u- of m >= 0 (those of -m are the other one's of m) and
+    // the imaginary part of u_z.
+    std::vector<double> hp(sys, 0.0), hm(sys, 0.0), hz(sys, 0.0);
+    const bool done = factor_tables(
+        h, h.fxH, h.facH, h.facHT, M + 2, [&](int ma, double kz) { return helmholtz_band(h, ma, kz); },
+        [&](int mu, int k, const std::vector<double>& f) {
+            const double kz = 2.0 * M_PI * k / d.Lz;
+            std::vector<double> x(nr);
+            auto solve = [&](int m, int kind, std::vector<double>& to) {  // kind +1, -1: u+-, 0: u_z
+                if (m < 0 || m > M || (m == 0 && k == 0)) return;
+                const double* phi = &h.phi[at(m, k)];
+                const int pp = parity_index(m);
+                for (int j = 0; j < nr; ++j) {
+                    if (kind == 0) {
+                        x[j] = -kz * phi[j];
+                        continue;
+                    }
+                    double dphi = 0;
+                    for (int c = std::max(0, j - kLo); c <= std::min(nr - 1, j + kUp); ++c)
+                        dphi += h.D1[((size_t)pp * nr + j) * kBand + (c - j + kLo)] * phi[c];
+                    x[j] = -dphi + kind * m * h.invr[j] * phi[j];
+                }
+                x[0] = 0.0;
+                band_solve(nr, f, x);
+                std::copy(x.begin(), x.end(), to.begin() + at(m, k));
+            };
+            solve(mu - 1, 1, hp);
+            solve(mu + 1, -1, hm);
+            if (mu == 1) solve(0, -1, hm);
+            solve(mu, 0, hz);
+        },
+        worst);
+    if (!done) {
+        err = "Helmholtz band LU failed";
+        return false;
+    }
     if (!(worst < 1e-12)) {
         char buf[160];
         std::snprintf(buf, sizeof buf, "banded LU without pivoting is unstable here (backward error %.3g)", worst);
         err = buf;
         return false;
     }
-    // influence responses: phi solves the pressure problem with a unit wall
-    // datum, h the Helmholtz response to -grad(phi) with u = 0 at the wall;
-    // stored scaled by -1/delta, delta = d/dr(h_r) at the wall.
+    // influence responses, stored scaled by -1/delta, delta = d/dr(h_r) at the
+    // wall; k fastest, [im][component][j][k], so that the device reads them
+    // coalesced across the k of a block
     h.infl.assign((size_t)d.nm * nk * 3 * nr, 0.0);
     std::vector<int> zero_t(16, 0);
-    parallel_k(nk, [&](int k, int t) {
-        std::vector<double> f, fac_tmp;
-        const double kz = 2.0 * M_PI * k / d.Lz;
-        for (int im = 0; im < d.nm; ++im) {
-            const int m = im - M;
+    const int nkt = (nk + kTileX - 1) / kTileX;
+    parallel_k((M + 1) * nkt, [&](int item, int t) {
+        const int m = item / nkt, k0 = item % nkt * kTileX, pv = parity_index(m + 1);
+        for (int k = k0; k < std::min(nk, k0 + kTileX); ++k) {
             if (m == 0 && k == 0) continue;
-            const int ma = std::abs(m);
-            gather_factors(h.facP, ma, k, nr, nt, D, f);  // factors computed above
-            std::vector<double> phi(nr, 0.0);
-            phi[0] = 1.0;
-            band_solve(nr, f, phi);
-            const int pp = parity_index(m);
-            std::vector<double> dphi(nr, 0.0);
-            for (int j = 0; j < nr; ++j)
-                for (int c = std::max(0, j - kLo); c <= std::min(nr - 1, j + kUp); ++c)
-                    dphi[j] += h.D1[((size_t)pp * nr + j) * kBand + (c - j + kLo)] * phi[c];
-            std::vector<double> fp(nr), fm(nr), fz(nr);
-            for (int j = 0; j < nr; ++j) {
-                fp[j] = -dphi[j] + m * h.invr[j] * phi[j];
-                fm[j] = -dphi[j] - m * h.invr[j] * phi[j];
-                fz[j] = -kz * phi[j];  // imaginary part of -i kz phi
-            }
-            fp[0] = fm[0] = fz[0] = 0.0;
-            gather_factors(h.facH, std::abs(m + 1), k, nr, nt, D, fac_tmp);
-            band_solve(nr, fac_tmp, fp);
-            gather_factors(h.facH, std::abs(m - 1), k, nr, nt, D, fac_tmp);
-            band_solve(nr, fac_tmp, fm);
-            gather_factors(h.facH, ma, k, nr, nt, D, fac_tmp);
-            band_solve(nr, fac_tmp, fz);
-            std::vector<double> hr(nr), hti(nr);
-            for (int j = 0; j < nr; ++j) {
-                hr[j] = 0.5 * (fp[j] + fm[j]);
-                hti[j] = -0.5 * (fp[j] - fm[j]);
-            }
-            const int pv = parity_index(m + 1);
+            const double *fp = &hp[at(m, k)], *fm = &hm[at(m, k)], *fz = &hz[at(m, k)];
             double delta = 0;
-            for (int c = 0; c <= kUp && c < nr; ++c) delta += h.D1[((size_t)pv * nr + 0) * kBand + (c + kLo)] * hr[c];
+            for (int c = 0; c <= kUp && c < nr; ++c)
+                delta += h.D1[((size_t)pv * nr + 0) * kBand + (c + kLo)] * (0.5 * (fp[c] + fm[c]));
             if (!(std::fabs(delta) > 1e-300) || !std::isfinite(delta)) {
                 zero_t[t] = 1;
                 return;
             }
-            // k fastest: [im][component][j][k], so that the device reads it
-            // coalesced across the k of a block
-            double* out = &h.infl[(size_t)im * 3 * nr * nk + k];
-            for (int j = 0; j < nr; ++j) {
-                out[(size_t)j * nk] = -hr[j] / delta;
-                out[((size_t)nr + j) * nk] = -hti[j] / delta;
-                out[((size_t)2 * nr + j) * nk] = -fz[j] / delta;
+            for (int side = 0; side < (m ? 2 : 1); ++side) {
+                double* out = &h.infl[(size_t)(side ? M - m : M + m) * 3 * nr * nk + k];
+                for (int j = 0; j < nr; ++j) {
+                    const double ht = -0.5 * (fp[j] - fm[j]);
+                    out[(size_t)j * nk] = -(0.5 * (fp[j] + fm[j])) / delta;
+                    out[((size_t)nr + j) * nk] = (side ? ht : -ht) / delta;
+                    out[((size_t)2 * nr + j) * nk] = -fz[j] / delta;
+                }
             }
         }
     });
@@ -497,11 +828,12 @@ bool build_operators(HostOps& h, std::string& err, bool reuse_pressure) {
         }
     // flux response of mode (0,0): Helmholtz of u_z with unit forcing
     {
-        Band Hz = helmholtz_band(h, 0, 0.0);
-        band_lu(Hz, fac_tmp, growth);
+        std::vector<double> f;
+        double growth = 0;
+        band_lu(helmholtz_band(h, 0, 0.0), f, growth);
         h.fluxg.assign(nr, 1.0);
         h.fluxg[0] = 0.0;
-        band_solve(nr, fac_tmp, h.fluxg);
+        band_solve(nr, f, h.fluxg);
         double s = 0;
         for (int j = 0; j < nr; ++j) s += h.W[j] * h.fluxg[j];
         h.flux_inv = 1.0 / s;

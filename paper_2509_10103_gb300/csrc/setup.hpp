@@ -42,6 +42,65 @@ inline size_t fac_index(int mat, int k, int j, int e, int nr, int ntile, int nc1
 constexpr int kNc1Direct = kLo;          // A x = b rows: l (4) | 1/diag, U (9)
 constexpr int kNc1Transposed = kUp + 1;  // A^T x = b rows: U^T (8), 1/diag | L^T (4)
 
+// Fixed-point factor table of the integer solver, which takes each system from
+// both ends at once.  The rows [0, h) and [h, nr) are eliminated towards h, up
+// to the four rows on either side of it; with those eight kept as one block S,
+//   A = N M:  N unit (multipliers of the outer rows), M = D U outside (U with a
+//   unit diagonal, coupling a row to the rows nearer h) and S in the middle.
+// A side counts its rows ("positions") from its end of the grid inwards, in
+// chunks of four; the last chunk is its half of the middle, and the inner side's
+// positions are shifted so that it is whole (empty positions at the axis).
+// The sweeps need, negated and in fixed point (58 fractional bits, kept as a
+// signed high and a signed low 32-bit digit), per position four multipliers of
+// N or U by row (direct) or by column (transposed).  A (matrix, tile of kTileX
+// k) holds, a 16-byte read being two multipliers of one k:
+//   side 0 then side 1:  inward, [chunk][4][2][k][2] (positions p-4..p-1);
+//     outward, [chunk but the last]: [4][2][k][2] (positions p+1..p+4) and 1/D as
+//     [4][k], a 62-bit fixed-point number whose low byte is its exponent, shared
+//     by the rows of a chunk but in the first one; the side's half of S^-1 (or
+//     its transpose), [4][4][k][2] (own four, then the other side's four, in
+//     positions) and its exponent, [k];
+//   the wider wall rows, [4][4][k]: columns 5..8 of rows 0..3 of U (direct), rows
+//     0..3 of U for columns 5..8 (transposed).
+// The wall row of A (Dirichlet or Neumann) is not scaled like the others, so
+// column 0 of N is large: it is stored times 2^-shift and its value enters the
+// window times 2^shift.  The solver's 64-bit sums need sum |multiplier| <=
+// kFxRowSum in every row; on the unstretched grid the sums stay below 4.0 for
+// the pressure and 2.5 for the Helmholtz matrices (24 to 128 points, any Re dt);
+// wide one-sided stencils of stretched grids can exceed it (62 at stretch 0.1).
+constexpr int kTileX = 16;
+constexpr int kFxBits = 58;
+constexpr double kFxRowSum = 6.0;
+constexpr int kFxMinRows = 21;  // smaller grids keep the FP64 solver
+struct FixedTable {
+    bool ok = false;
+    int shift = 0;
+    std::vector<double> direct, transposed;
+};
+struct FxShape {
+    int h, chunks[2], pad;  // rows of side 0, chunks of the sides, empty positions of side 1
+    size_t in[2], out[2], mid[2], wall, tile;  // offsets in a tile (8-byte words), its size
+};
+inline FxShape fx_shape(int nr) {
+    FxShape f;
+    f.h = 4 * ((nr + 4) / 8 > 4 ? (nr + 4) / 8 : 4);
+    const int lower = nr - f.h > 0 ? nr - f.h : 0;
+    f.chunks[0] = f.h / 4;
+    f.chunks[1] = (lower + 3) / 4;
+    f.pad = 4 * f.chunks[1] - lower;
+    size_t at = 0;
+    for (int s = 0; s < 2; ++s) {
+        const size_t n = f.chunks[s], outer = n > 0 ? n - 1 : 0;
+        f.in[s] = at;
+        f.out[s] = f.in[s] + n * 16 * kTileX;
+        f.mid[s] = f.out[s] + outer * 20 * kTileX;
+        at = f.mid[s] + 33 * kTileX;
+    }
+    f.wall = at;
+    f.tile = f.wall + 16 * kTileX;
+    return f;
+}
+
 // Everything the device needs, laid out for coalesced access across k.
 struct HostOps {
     Dims d;
@@ -49,13 +108,16 @@ struct HostOps {
     std::vector<double> r, invr, W;            // [nr]
     std::vector<double> D1, D2;                 // [2 parity][nr][kBand], parity 0 even, 1 odd
     std::vector<double> Lb;                     // [M+2][nr][kBand]  D2 + D1/r - m^2/r^2 (no kz^2)
-    // Banded LU factors in the tiled layout of fac_index (ntile tiles of k,
-    // zeros beyond nk).  Row layout "lower | 1/diag | upper" for a two-sweep solve:
+    // Banded factors for the device: fixed-point tables of M+2 Helmholtz
+    // matrices (per |m'|, k) and M+1 pressure matrices (per |m|, k), or where a
+    // row's multipliers do not fit (ok false) FP64 rows in the tiled layout of
+    // fac_index (ntile tiles of k, zeros beyond nk), "lower | 1/diag | upper":
     //   facH/facP  (A x = b):   l_{j,j-4..j-1}, 1/U_jj, U_{j,j+1..j+8}    (nc1 = kNc1Direct)
     //   facHT/facPT (A^T x = b): U_{j-8..j-1,j}, 1/U_jj, L_{j+1..j+4,j}  (nc1 = kNc1Transposed)
     int ntile = 0;
-    std::vector<double> facH, facHT;            // M+2 matrices (per |m'|, k)  Helmholtz
-    std::vector<double> facP, facPT;            // M+1 matrices (per |m|, k)   pressure
+    FixedTable fxH, fxP;
+    std::vector<double> facH, facHT, facP, facPT;
+    std::vector<double> phi;                    // [M+1][nk][nr] pressure of a unit wall datum
     std::vector<double> infl;                   // [nm][3][nr][nk] influence response, pre-scaled by -1/delta
     std::vector<double> fluxg;                  // [nr] flux response of mode (0,0)
     double flux_inv = 0;                        // 1 / sum_j W_j g_j
@@ -68,8 +130,8 @@ int parity_index(int m);  // 0 when m is even, 1 when odd
 // Builds grid, weights and finite differences (Re-independent part).
 bool build_grid(HostOps& h, std::string& err);
 // Builds base flow, banded LU factors, influence and flux vectors.
-// reuse_pressure: keep h.facP / h.facPT when they already have this grid's
-// size (they depend on the grid only, not on Re or dt).
+// reuse_pressure: keep h.phi, and leave the pressure tables alone, when it
+// already has this grid's size (they depend on the grid only, not on Re or dt).
 bool build_operators(HostOps& h, std::string& err, bool reuse_pressure = false);
 
 // Bessel J_nu of complex argument by its power series.
