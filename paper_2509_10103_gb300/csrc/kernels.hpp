@@ -89,10 +89,13 @@ struct ZScales {
     float fh0[kMaxIn], fhk[kMaxIn], fo0[6], fok[6];  // FP32 copies, filled by launch_zpass
 };
 
-// Twiddle tables e^{-2 pi i n / N} for N = nt and N = nzp, FP64 and FP32.
+// Twiddle tables e^{-2 pi i n / N} for N = nt and N = nzp: FP32, FP64 (z only)
+// and in fixed point (62 fractional bits; low and high signed 32-bit digit of the real
+// part, then of the imaginary part).
 struct Twiddles {
-    const double2* th_d;
     const double2* z_d;
+    const int4* th_x;
+    const int4* z_x;
     const float2* th_f;
     const float2* z_f;
 };

@@ -243,6 +243,23 @@ template <class T2> std::vector<T2> twiddle_table(int N) {
     return t;
 }
 
+// the same in fixed point (see Twiddles)
+std::vector<int4> twiddle_digits(int N) {
+    std::vector<int4> t(N);
+    auto digits = [](long double v, int& lo, int& hi) {
+        long long c = std::llround(std::ldexp(v, 62));
+        if ((unsigned)(c & 0xFFFFFFFFll) == 0x80000000u) ++c;  // a digit that can be negated
+        lo = (int)(unsigned)(c & 0xFFFFFFFFll);
+        hi = (int)((c - lo) >> 32);
+    };
+    for (int n = 0; n < N; ++n) {
+        const long double a = -2.0L * 3.14159265358979323846264338327950288L * n / N;
+        digits(std::cos(a), t[n].x, t[n].y);
+        digits(std::sin(a), t[n].z, t[n].w);
+    }
+    return t;
+}
+
 // Tables of slot `slot` from the operators h was built with (Re, dt, Wo and
 // A of that slot's request).  The per-slot tables are allocated for all slots
 // on first use; the grid-only tables (pressure factors) are written once.
@@ -1704,10 +1721,13 @@ int create_impl(const pnop_grid* grid, const pnop_params* params, void* cuda_str
             }
         }
         upload_operators(c);
-        auto thd = twiddle_table<double2>(d.nth), zd = twiddle_table<double2>(d.nzp);
+        auto zd = twiddle_table<double2>(d.nzp);
         auto thf = twiddle_table<float2>(d.nth), zf = twiddle_table<float2>(d.nzp);
-        c->tw.th_d = c->upload(thd);
         c->tw.z_d = c->upload(zd);
+        if (!mixed(c)) {
+            c->tw.th_x = c->upload(twiddle_digits(d.nth));
+            c->tw.z_x = c->upload(twiddle_digits(d.nzp));
+        }
         c->tw.th_f = c->upload(thf);
         c->tw.z_f = c->upload(zf);
         for (double2** b : {&c->omega, &c->N0, &c->N1, &c->us, &c->ua, &c->Fb, &c->Nb, &c->ubs, &c->wb, &c->R,

@@ -5,9 +5,11 @@
 // carry the batch entry in the grid's z dimension (with the field index for
 // the theta kernels) and offset spectral and physical buffers by its slot.
 #include "dev_common.cuh"
+#include "dev_x64.cuh"
 #include "kernels.hpp"
 
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 #include <utility>
 
@@ -271,6 +273,428 @@ __global__ void k_zpass(Geo g, const T2* __restrict__ Y, T2* __restrict__ Z, ZSc
             T2 z2 = mk<T2>((T)0.5 * (P.y + Pm.y) * s2, (T)-0.5 * (P.x - Pm.x) * s2);
             Z[((size_t)(o2 * g.nr + j) * g.nt + a) * nk + k] = z2;
         }
+    }
+}
+
+// ------------------------------------------------------------------ fixed-point transforms
+// The FP64 transforms run in 64-bit fixed point (dev_x64.cuh): an FP64 addition
+// takes 77 cycles of its pipe, a 64-bit integer one about 2, and a product by a
+// twiddle factor (62 fractional bits) four IMAD.WIDE of 4.2.  The values of a
+// transform share one exponent.  For spectra it is chosen from the sum of the
+// magnitudes of the inputs, which bounds every intermediate result: a unit is
+// 2^-60 of that sum.  The forward z transform takes its values, products of
+// physical fields, at full length and halves them as often as a stage can double
+// them (SCALE).  Nothing can wrap either way.
+struct fx2 {
+    long long x, y;
+};
+constexpr int kXT = 62;  // fractional bits of a twiddle factor
+__device__ __forceinline__ fx2 fx_add(fx2 a, fx2 b) { return {a.x + b.x, a.y + b.y}; }
+__device__ __forceinline__ fx2 fx_sub(fx2 a, fx2 b) { return {a.x - b.x, a.y - b.y}; }
+// (a c + b s) 2^-SH with multipliers of kXT fractional bits, |c|, |s| <= 1, |a|, |b| < 2^61
+template <int SH> __device__ __forceinline__ long long fx_dot2(xdig a, int2 c, xdig b, int2 s) {
+    long long m = x_mad(s.y, b.l, x_mad(s.x, b.h, x_mad(c.y, a.l, x_mad(c.x, a.h, 1ll << (kXT - 33 + SH)))));
+    const long long l0 = x_mul(c.x, a.l), l1 = x_mul(s.x, b.l), h = x_mad(s.y, b.h, x_mul(c.y, a.h));
+    m += (long long)(int)(l0 >> 32) + (long long)(int)(l1 >> 32);
+    return (h << (64 - kXT - SH)) + (m >> (kXT - 32 + SH));
+}
+// v e^{SIGN i phi} 2^-SH, w = (cos, -sin) of phi
+template <int SIGN, int SH> __device__ __forceinline__ fx2 fx_rot(fx2 v, int4 w) {
+    const xdig x = x_split(v.x), y = x_split(v.y);
+    const int2 c = make_int2(w.x, w.y), s = make_int2(w.z, w.w), ns = make_int2(-w.z, -w.w);
+    // e^{-i phi} = c + i s: (x c - y s, y c + x s); e^{+i phi} = c - i s
+    return SIGN < 0 ? fx2{fx_dot2<SH>(x, c, y, ns), fx_dot2<SH>(y, c, x, s)}
+                    : fx2{fx_dot2<SH>(x, c, y, s), fx_dot2<SH>(y, c, x, ns)};
+}
+template <int R, int SIGN> __device__ __forceinline__ void fx_dft(fx2* v) {
+    if (R == 2) {
+        const fx2 a = v[0], b = v[1];
+        v[0] = fx_add(a, b);
+        v[1] = fx_sub(a, b);
+    } else if (R == 4) {
+        const fx2 s02 = fx_add(v[0], v[2]), d02 = fx_sub(v[0], v[2]), s13 = fx_add(v[1], v[3]), d13 = fx_sub(v[1], v[3]);
+        const fx2 id = SIGN > 0 ? fx2{-d13.y, d13.x} : fx2{d13.y, -d13.x};
+        v[0] = fx_add(s02, s13);
+        v[2] = fx_sub(s02, s13);
+        v[1] = fx_add(d02, id);
+        v[3] = fx_sub(d02, id);
+    } else {  // R == 3
+        constexpr long long h = 3993837246235628775ll;  // sqrt(3)/2 2^62
+        const int2 hd = make_int2((int)(unsigned)(h & 0xFFFFFFFFll), (int)((h + (1ll << 31)) >> 32));
+        const fx2 t1 = fx_add(v[1], v[2]), d = fx_sub(v[1], v[2]);
+        const fx2 t2 = {v[0].x - (t1.x >> 1), v[0].y - (t1.y >> 1)};
+        const long long px = x_prod<kXT>(hd, x_split(d.x), 1ll << (kXT - 33)), py = x_prod<kXT>(hd, x_split(d.y), 1ll << (kXT - 33));
+        const fx2 t3 = SIGN > 0 ? fx2{-py, px} : fx2{py, -px};
+        v[0] = fx_add(v[0], t1);
+        v[1] = fx_add(t2, t3);
+        v[2] = fx_sub(t2, t3);
+    }
+}
+// the Stockham stages of fft_cols in fixed point
+template <int R, int NCOL, int LD, int SIGN, bool SCALE>
+__device__ __forceinline__ void fx_stage(const fx2* __restrict__ a, fx2* __restrict__ b, int N, int Ns, int lgNs,
+                                         const int4* __restrict__ tw) {
+    constexpr int SH = !SCALE ? 0 : (R == 2 ? 1 : 2);  // what the stage can grow by (the first stage is not scaled)
+    const int stride = N / R, nb = stride * NCOL, tstep = N / (Ns * R);
+    for (int idx = threadIdx.x; idx < nb; idx += blockDim.x) {
+        const int col = idx % NCOL, jb = idx / NCOL;
+        int q, kk;
+        if (lgNs >= 0) {
+            q = jb >> lgNs;
+            kk = jb & (Ns - 1);
+        } else {
+            q = jb / Ns;
+            kk = jb - q * Ns;
+        }
+        fx2 v[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = a[(jb + r * stride) * LD + col];
+        if (Ns > 1) {
+            const int tb = kk * tstep;
+#pragma unroll
+            for (int r = 1; r < R; ++r) v[r] = fx_rot<SIGN, SH>(v[r], tw[r * tb]);
+            if (SCALE) v[0] = {(v[0].x + SH) >> SH, (v[0].y + SH) >> SH};  // SH = 1 or 2: half a unit is SH
+        }
+        fx_dft<R, SIGN>(v);
+        const int idxD = q * Ns * R + kk;
+#pragma unroll
+        for (int r = 0; r < R; ++r) b[(idxD + r * Ns) * LD + col] = v[r];
+    }
+}
+// halvings: what the result is to be multiplied by, as an exponent of 2 (SCALE)
+template <int NCOL, int LD, int SIGN, bool SCALE = false>
+__device__ fx2* fx_cols(fx2* a, fx2* b, int N, const int4* tw, int* halvings = nullptr) {
+    const int n2 = __ffs(N) - 1;
+    int n3 = 0;
+    for (int t = N >> n2; t > 1; t /= 3) ++n3;
+    int Ns = 1, lgNs = 0;
+    auto next = [&](int R) {
+        __syncthreads();
+        fx2* t = a;
+        a = b;
+        b = t;
+        if (SCALE && Ns > 1) *halvings += R == 2 ? 1 : 2;
+        Ns *= R;
+    };
+    for (int st = 0; st < n2 / 2; ++st) {
+        fx_stage<4, NCOL, LD, SIGN, SCALE>(a, b, N, Ns, lgNs, tw);
+        next(4);
+        lgNs += 2;
+    }
+    if (n2 & 1) {
+        fx_stage<2, NCOL, LD, SIGN, SCALE>(a, b, N, Ns, lgNs, tw);
+        next(2);
+        lgNs += 1;
+    }
+    for (int st = 0; st < n3; ++st) {
+        fx_stage<3, NCOL, LD, SIGN, SCALE>(a, b, N, Ns, st == 0 ? lgNs : -1, tw);
+        next(3);
+    }
+    return a;
+}
+// magnitude of x relative to 2^top as a count of 2^-19, rounded up (0 for zero);
+// top: the exponent field of the largest value
+__device__ __forceinline__ unsigned fx_count(double x, int top) {
+    const int h = __double2hiint(x) & 0x7FFFFFFF, e = h >> 20;
+    return e ? ((((unsigned)h & 0xFFFFFu) | 0x100000u) >> min(top - e + 1, 31)) + 1u : 0u;
+}
+// unit (as an exponent of 2) in which values sum to less than 2^bits, `sum` being
+// the sum of their counts in steps of four
+__device__ __forceinline__ int fx_unit(unsigned sum, int top, int bits) {
+    return top - 1023 - 17 + (32 - __clz((int)sum)) - bits;
+}
+__device__ __forceinline__ int x_top(long long v) { return 64 - __clzll(v ^ (v >> 63)); }  // |v| <= 2^top
+
+// the z pass in fixed point: contract of k_zpass (FP64), any length.  The fields
+// fall into the groups u, w and (modes ZADJ, ZCADJ) g, each with one unit; a
+// group's input scale is gs for k = 0 and gs hs for k > 0, hs a power of two (hsh
+// its exponent), and gs is part of the output scales o0, ok.
+struct XScales {
+    int hsh[3];
+    double o0[6], ok[6];
+};
+template <int MODE>
+__global__ void k_zpass_x(Geo g, const double2* __restrict__ Y, double2* __restrict__ Z, XScales sc,
+                          const int4* __restrict__ twg) {
+    grid_dep_sync();
+    constexpr int NIN = MODE == ZFWD ? 6 : 9;
+    constexpr int NPI = (NIN + 1) / 2;
+    constexpr int NOUT = MODE == ZADJ ? 6 : 3;
+    constexpr int NPO = (NOUT + 1) / 2;
+    constexpr int NG = NIN / 3;
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int top_sh[3], max_sh[3];
+    __shared__ unsigned sum_sh[NIN];
+    const int N = g.nzp, nk = g.nk;
+    fx2* bufA = reinterpret_cast<fx2*>(smem);
+    fx2* bufB = bufA + N * NPI;
+    int4* tw = reinterpret_cast<int4*>(bufB + N * NPI);
+    const int a = blockIdx.x, j = blockIdx.y;
+    const size_t poff = (size_t)g.slot[blockIdx.z] * g.ps;
+    Y += poff;
+    Z += poff;
+    if (threadIdx.x < 3) top_sh[threadIdx.x] = max_sh[threadIdx.x] = 0;
+    if (threadIdx.x < NIN) sum_sh[threadIdx.x] = 0;
+    for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = twg[i];
+    __syncthreads();
+    // inputs into bufB as they are, the largest exponent of each group
+    double2* raw = reinterpret_cast<double2*>(bufB);  // [NIN][nk]
+    {
+        int mx[NG] = {};
+#pragma unroll
+        for (int f = 0; f < NIN; ++f)
+            for (int k = threadIdx.x; k < nk; k += blockDim.x) {
+                double2 y = Y[((size_t)(f * g.nr + j) * g.nt + a) * nk + k];
+                if (k == 0) y.y = 0;
+                raw[f * nk + k] = y;
+                mx[f / 3] = max(mx[f / 3], max(__double2hiint(y.x) & 0x7FFFFFFF, __double2hiint(y.y) & 0x7FFFFFFF));
+            }
+#pragma unroll
+        for (int i = 0; i < NG; ++i) {
+            const int m = __reduce_max_sync(0xffffffffu, mx[i]);
+            if ((threadIdx.x & 31) == 0) atomicMax(&top_sh[i], m);
+        }
+    }
+    __syncthreads();
+    bool bad = false;
+    int top[NG];
+#pragma unroll
+    for (int i = 0; i < NG; ++i) {
+        bad = bad || top_sh[i] >= 0x7FF00000;
+        top[i] = top_sh[i] >> 20;
+    }
+#pragma unroll
+    for (int f = 0; f < NIN; ++f) {
+        unsigned s = 0;
+        for (int k = threadIdx.x; k < nk; k += blockDim.x) {
+            const double2 y = raw[f * nk + k];
+            s += (fx_count(y.x, top[f / 3]) + fx_count(y.y, top[f / 3]) + 3u) >> 2;  // nk up to 2^12
+        }
+        s = __reduce_add_sync(0xffffffffu, s);
+        if ((threadIdx.x & 31) == 0) atomicAdd(&sum_sh[f], s);
+    }
+    __syncthreads();
+    int E[NG];  // |f| <= 2 sum of the magnitudes < 2^60 units; a packed column < 2^61
+#pragma unroll
+    for (int i = 0; i < NG; ++i)
+        E[i] = max(fx_unit(max(sum_sh[3 * i], max(sum_sh[3 * i + 1], sum_sh[3 * i + 2])), top[i], 59), -kXTop);
+    // Hermitian-extended spectra, two fields per column
+    for (int n = threadIdx.x; n < NPI * (N - 2 * nk + 1); n += blockDim.x) bufA[nk * NPI + n] = {0, 0};
+#pragma unroll
+    for (int p = 0; p < NPI; ++p) {
+        constexpr int none = NIN;
+        const int f1 = 2 * p, f2 = 2 * p + 1 < NIN ? 2 * p + 1 : none, g1 = f1 / 3, g2 = f2 == none ? g1 : f2 / 3;
+        const xunit u1 = x_unit(E[g1]), u2 = x_unit(E[g2]);
+        for (int k = threadIdx.x; k < nk; k += blockDim.x) {
+            const double2 y1 = raw[f1 * nk + k], y2 = f2 == none ? make_double2(0, 0) : raw[f2 * nk + k];
+            fx2 h1 = {x_load(y1.x, u1), x_load(y1.y, u1)}, h2 = {0, 0};
+            if (f2 != none) h2 = {x_load(y2.x, u2), x_load(y2.y, u2)};
+            if (k > 0 && MODE == ZADJ) {
+                h1 = {h1.x >> sc.hsh[g1], h1.y >> sc.hsh[g1]};
+                h2 = {h2.x >> sc.hsh[g2], h2.y >> sc.hsh[g2]};
+            }
+            bufA[k * NPI + p] = {h1.x - h2.y, h1.y + h2.x};                    // H1 + i H2
+            if (k > 0) bufA[(N - k) * NPI + p] = {h1.x + h2.y, h2.x - h1.y};  // conj(H1) + i conj(H2)
+        }
+    }
+    __syncthreads();
+    fx2* ph = fx_cols<NPI, NPI, +1>(bufA, bufB, N, tw);
+    fx2* pr = ph == bufA ? bufB : bufA;
+    // largest physical values of the groups, for the units of the products
+    {
+        long long mx[3] = {};
+        for (int n = threadIdx.x; n < N; n += blockDim.x) {
+            const long long* row = reinterpret_cast<const long long*>(ph + n * NPI);
+#pragma unroll
+            for (int f = 0; f < NIN; ++f) mx[f / 3] |= row[f] ^ (row[f] >> 63);
+        }
+#pragma unroll
+        for (int i = 0; i < NG; ++i) {
+            const int m = __reduce_max_sync(0xffffffffu, x_top(mx[i]));
+            if ((threadIdx.x & 31) == 0) atomicMax(&max_sh[i], m);
+        }
+    }
+    __syncthreads();
+    // a product (a b - c d) is shifted by 60 + sh, so that two of them stay below
+    // 2^59 (the first stage of the forward transform at most quadruples them)
+    auto shift = [&](int ga, int gb) { return max(max_sh[ga] + max_sh[gb] + 2 - 60 - 59, 0); };
+    auto cross = [&](xdig p, xdig q, xdig nr, xdig t, int sh) {  // (p q + nr t) >> (60 + sh)
+        long long m = x_mad(nr.h, t.l, x_mad(nr.l, t.h, x_mad(p.h, q.l, x_mul(p.l, q.h))));
+        const long long l0 = x_mul(p.l, q.l), l1 = x_mul(nr.l, t.l), h = x_mad(nr.h, t.h, x_mul(p.h, q.h));
+        m += (long long)(int)(l0 >> 32) + (long long)(int)(l1 >> 32);
+        return ((h << 4) + (m >> 28)) >> sh;
+    };
+    const int s01 = shift(0, 1), s12 = MODE == ZADJ ? shift(1, 2) : 0, s02 = MODE == ZADJ ? shift(0, 2) : 0;
+    for (int n = threadIdx.x; n < N; n += blockDim.x) {
+        const long long* row = reinterpret_cast<const long long*>(ph + n * NPI);
+        xdig v[NIN], n_[NIN];  // digits of the values and of their negatives
+#pragma unroll
+        for (int f = 0; f < NIN; ++f) {
+            v[f] = x_split(row[f]);
+            n_[f] = x_split(-row[f]);
+        }
+        fx2* o = pr + n * NPI;
+        if (MODE == ZFWD) {  // u x w
+            o[0] = {cross(v[1], v[5], n_[2], v[4], s01), cross(v[2], v[3], n_[0], v[5], s01)};
+            o[1] = {cross(v[0], v[4], n_[1], v[3], s01), 0};
+        } else {  // w x g, g x u
+            constexpr int g0 = NIN - 3;
+            o[0] = {cross(v[4], v[g0 + 2], n_[5], v[g0 + 1], s12), cross(v[5], v[g0], n_[3], v[g0 + 2], s12)};
+            o[1] = {cross(v[3], v[g0 + 1], n_[4], v[g0], s12), cross(v[g0 + 1], v[2], n_[1], v[g0 + 2], s02)};
+            o[2] = {cross(v[g0 + 2], v[0], n_[2], v[g0], s02), cross(v[g0], v[1], n_[0], v[g0 + 1], s02)};
+        }
+    }
+    __syncthreads();
+    int halvings = 0;
+    fx2* sp = fx_cols<NPO, NPI, -1, true>(pr, ph, N, tw, &halvings);
+    const int nan = bad ? 0x7FF80000 : 0;
+    int Eo[2];  // units of the products of the first three outputs and of the others, times 1/2 of the separation
+    Eo[0] = (MODE == ZFWD ? E[0] + E[1] + s01 : E[1] + E[NG - 1] + s12) + 60 - 1 + halvings;
+    Eo[1] = E[0] + E[NG - 1] + s02 + 60 - 1 + halvings;
+    const bool far = Eo[0] < -1000 || Eo[0] > 900 || Eo[1] < -1000 || Eo[1] > 900;
+    auto put = [&](int f, int k, long long x, long long y) {
+        const int e = Eo[f / 3];
+        const double s = k == 0 ? sc.o0[f] : sc.ok[f];
+        double2 z;
+        if (far) z = make_double2(x_store_any(x, e, nan) * s, x_store_any(y, e, nan) * s);
+        else z = make_double2(x_store(x, e, nan) * s, x_store(y, e, nan) * s);
+        Z[((size_t)(f * g.nr + j) * g.nt + a) * nk + k] = z;
+    };
+#pragma unroll
+    for (int p = 0; p < NPO; ++p)
+        for (int k = threadIdx.x; k < nk; k += blockDim.x) {
+            const fx2 P = sp[k * NPI + p], Q = sp[(k ? N - k : 0) * NPI + p];
+            put(2 * p, k, P.x + Q.x, P.y - Q.y);
+            if (2 * p + 1 < NOUT) put(2 * p + 1, k, P.y + Q.y, Q.x - P.x);
+        }
+}
+
+// The theta transforms in fixed point, any length: contract of k_synth_theta and
+// k_anal_theta (FP64).  A block takes KB columns k of one (field, j), all in one
+// unit (the z pass sums over k, so a column far below its neighbours does not
+// count there).  Rows of `in` values from memory into `raw`, and the unit in
+// which the magnitudes of every column sum to less than 2^61; bad: infinities or NaN.
+template <int KB, class F>
+__device__ __forceinline__ int fx_columns(int rows, int kw, double2* raw, F&& load, int* top_sh, unsigned* sum_sh, bool& bad) {
+    const int kk = threadIdx.x % KB, r0 = threadIdx.x / KB, dr = blockDim.x / KB;  // a thread keeps to one column
+    if (threadIdx.x == 0) *top_sh = 0;
+    if (threadIdx.x < KB) sum_sh[threadIdx.x] = 0;
+    __syncthreads();
+    int mx = 0;
+    for (int r = r0; r < rows; r += dr) {
+        const double2 y = kk < kw ? load(r, kk) : make_double2(0, 0);
+        raw[r * KB + kk] = y;
+        mx = max(mx, max(__double2hiint(y.x) & 0x7FFFFFFF, __double2hiint(y.y) & 0x7FFFFFFF));
+    }
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if ((threadIdx.x & 31) == 0) atomicMax(top_sh, mx);
+    __syncthreads();
+    mx = *top_sh;
+    bad = mx >= 0x7FF00000;
+    const int top = mx >> 20;
+    unsigned s = 0;
+    for (int r = r0; r < rows; r += dr) {
+        const double2 y = raw[r * KB + kk];
+        s += (fx_count(y.x, top) + fx_count(y.y, top) + 3u) >> 2;
+    }
+    atomicAdd(&sum_sh[kk], s);
+    __syncthreads();
+    s = 0;
+#pragma unroll
+    for (int i = 0; i < KB; ++i) s = max(s, sum_sh[i]);
+    return max(fx_unit(s, top, 61), -kXTop);
+}
+__device__ __forceinline__ double2 fx_out(fx2 v, int E, bool far, int nan) {
+    return far ? make_double2(x_store_any(v.x, E, nan), x_store_any(v.y, E, nan))
+               : make_double2(x_store(v.x, E, nan), x_store(v.y, E, nan));
+}
+
+template <int KB>
+__global__ void k_synth_x(Geo g, FieldPtrs f, double2* __restrict__ Y, const int4* __restrict__ twg) {
+    grid_dep_sync();
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int top_sh;
+    __shared__ unsigned sum_sh[KB];
+    fx2* buf0 = reinterpret_cast<fx2*>(smem);
+    fx2* buf1 = buf0 + g.nt * KB;
+    int4* tw = reinterpret_cast<int4*>(buf1 + g.nt * KB);
+    const int k0 = blockIdx.x * KB, j = blockIdx.y;
+    const int nf = gridDim.z / g.nb, b = blockIdx.z / nf, fi = blockIdx.z - b * nf, slot = g.slot[b];
+    Y += (size_t)slot * g.ps;
+    const int kw = min(KB, g.nk - k0);
+    for (int i = threadIdx.x; i < g.nt; i += blockDim.x) tw[i] = twg[i];
+    const double2* src = f.in[fi] + (size_t)slot * g.fs + (size_t)j * g.nm * g.nk + k0;
+    double2* raw = reinterpret_cast<double2*>(buf1);
+    bool bad;
+    const int E = fx_columns<KB>(g.nm, kw, raw, [&](int r, int kk) { return src[(size_t)r * g.nk + kk]; }, &top_sh, sum_sh, bad);
+    const xunit u = x_unit(E);
+    for (int i = threadIdx.x; i < g.nt * KB; i += blockDim.x) {
+        const int n = i / KB, m = n <= g.M ? n : n - g.nt;  // zero-padded beyond |m| <= M
+        fx2 v = {0, 0};
+        if (m >= -g.M) {
+            const double2 y = raw[(m + g.M) * KB + i % KB];
+            v = {x_load(y.x, u), x_load(y.y, u)};
+        }
+        buf0[i] = v;
+    }
+    __syncthreads();
+    const fx2* res = fx_cols<KB, KB, +1>(buf0, buf1, g.nt, tw);
+    const int nan = bad ? 0x7FF80000 : 0;
+    const bool far = E < -1000 || E > 900;
+    double2* dst = Y + ((size_t)(fi * g.nr + j) * g.nt) * g.nk + k0;
+    for (int i = threadIdx.x; i < g.nt * KB; i += blockDim.x) {
+        const int a = i / KB, kk = i % KB;
+        if (kk < kw) dst[(size_t)a * g.nk + kk] = fx_out(res[i], E, far, nan);
+    }
+}
+
+template <int KB>
+__global__ void k_anal_x(Geo g, FieldPtrs f, const double2* __restrict__ Z, const int4* __restrict__ twg) {
+    grid_dep_sync();
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int top_sh;
+    __shared__ unsigned sum_sh[KB];
+    fx2* buf0 = reinterpret_cast<fx2*>(smem);
+    fx2* buf1 = buf0 + g.nt * KB;
+    int4* tw = reinterpret_cast<int4*>(buf1 + g.nt * KB);
+    const int k0 = blockIdx.x * KB, j = blockIdx.y;
+    const int nf = gridDim.z / g.nb, b = blockIdx.z / nf, fi = blockIdx.z - b * nf, slot = g.slot[b];
+    Z += (size_t)slot * g.ps;
+    const int kw = min(KB, g.nk - k0);
+    for (int i = threadIdx.x; i < g.nt; i += blockDim.x) tw[i] = twg[i];
+    const double2* src = Z + ((size_t)(fi * g.nr + j) * g.nt) * g.nk + k0;
+    double2* raw = reinterpret_cast<double2*>(buf1);
+    bool bad;
+    const int E = fx_columns<KB>(g.nt, kw, raw, [&](int r, int kk) { return src[(size_t)r * g.nk + kk]; }, &top_sh, sum_sh, bad);
+    const xunit u = x_unit(E);
+    for (int i = threadIdx.x; i < g.nt * KB; i += blockDim.x) {
+        const double2 y = raw[i];
+        buf0[i] = {x_load(y.x, u), x_load(y.y, u)};
+    }
+    __syncthreads();
+    const fx2* res = fx_cols<KB, KB, -1>(buf0, buf1, g.nt, tw);
+    const int nan = bad ? 0x7FF80000 : 0;
+    const bool far = E < -1000 || E > 900;
+    const size_t base = (size_t)slot * g.fs + (size_t)j * g.nm * g.nk + k0;
+    double2* dst = f.out[fi] + base;
+    const double2* add = f.add[fi] ? f.add[fi] + base : nullptr;
+    for (int i = threadIdx.x; i < g.nm * KB; i += blockDim.x) {
+        const int im = i / KB, kk = i % KB, m = im - g.M;
+        if (kk >= kw) continue;
+        const size_t o = (size_t)im * g.nk + kk;
+        fx2 v = res[(m < 0 ? m + g.nt : m) * KB + kk];
+        int e = E;
+        if (k0 + kk == 0) {  // Hermitian part
+            const fx2 w = res[(m > 0 ? g.nt - m : -m) * KB + kk];
+            v = {v.x + w.x, v.y - w.y};
+            e = E - 1;
+        }
+        double2 z = fx_out(v, e, far, nan);
+        if (add) {
+            const double2 y = add[o];
+            z = make_double2(z.x + y.x, z.y + y.y);
+        }
+        dst[o] = z;
     }
 }
 
@@ -799,9 +1223,6 @@ __global__ void __launch_bounds__(96, 6)
 }
 
 // ------------------------------------------------------------------ launchers
-template <class T2> static const T2* tw_theta(const Twiddles& t);
-template <> const double2* tw_theta<double2>(const Twiddles& t) { return t.th_d; }
-template <> const float2* tw_theta<float2>(const Twiddles& t) { return t.th_f; }
 template <class T2> static const T2* tw_z(const Twiddles& t);
 template <> const double2* tw_z<double2>(const Twiddles& t) { return t.z_d; }
 template <> const float2* tw_z<float2>(const Twiddles& t) { return t.z_f; }
@@ -846,38 +1267,78 @@ static void anal2(const Geo& g, const FieldPtrs& f, int nfield, const T2* Z, con
     launch_pdl(k_anal2<T2, KB, N1, N2>, grid, kT2, sm, s, g, f, Z, tw);
 }
 
+// columns per block of the fixed-point theta kernels: about 50 KB of shared
+// memory, 128 to 256 contiguous bytes per row
+static int theta_kx(const Geo& g) { return g.nt <= 96 && g.nk > 8 ? 16 : (g.nt <= 192 ? 8 : 4); }
+template <int KB> static size_t theta_sx(const Geo& g) { return (size_t)(2 * g.nt * KB + g.nt) * sizeof(double2); }
+static unsigned theta_tx(const Geo& g, int kb) {
+    return (unsigned)std::max(64, std::min(256, (g.nt * kb / 4 + 31) / 32 * 32));
+}
+template <int KB>
+static void synth_x(const Geo& g, const FieldPtrs& f, int nfield, double2* Y, const int4* tw, cudaStream_t s) {
+    smem_limit((const void*)k_synth_x<KB>);
+    launch_pdl(k_synth_x<KB>, dim3((g.nk + KB - 1) / KB, g.nr, nfield * g.nb), theta_tx(g, KB), theta_sx<KB>(g), s, g, f,
+               Y, tw);
+}
+template <int KB>
+static void anal_x(const Geo& g, const FieldPtrs& f, int nfield, const double2* Z, const int4* tw, cudaStream_t s) {
+    smem_limit((const void*)k_anal_x<KB>);
+    launch_pdl(k_anal_x<KB>, dim3((g.nk + KB - 1) / KB, g.nr, nfield * g.nb), theta_tx(g, KB), theta_sx<KB>(g), s, g, f,
+               Z, tw);
+}
+
 template <class T2>
 void launch_synth_theta(const Geo& g, const FieldPtrs& f, int nfield, T2* Y, const Twiddles& tw, cudaStream_t s) {
+    if constexpr (std::is_same<T2, double2>::value) {
+        switch (theta_kx(g)) {
+            case 16: synth_x<16>(g, f, nfield, Y, tw.th_x, s); break;
+            case 8: synth_x<8>(g, f, nfield, Y, tw.th_x, s); break;
+            default: synth_x<4>(g, f, nfield, Y, tw.th_x, s); break;
+        }
+        check_launch("synth_theta");
+        return;
+    } else {
     switch (g.nt) {
-        case 96: synth2<T2, 32, 8, 12>(g, f, nfield, Y, tw_theta<T2>(tw), s); check_launch("synth_theta"); return;
-        case 192: synth2<T2, 32, 16, 12>(g, f, nfield, Y, tw_theta<T2>(tw), s); check_launch("synth_theta"); return;
-        case 384: synth2<T2, 16, 16, 24>(g, f, nfield, Y, tw_theta<T2>(tw), s); check_launch("synth_theta"); return;
+        case 96: synth2<T2, 32, 8, 12>(g, f, nfield, Y, tw.th_f, s); check_launch("synth_theta"); return;
+        case 192: synth2<T2, 32, 16, 12>(g, f, nfield, Y, tw.th_f, s); check_launch("synth_theta"); return;
+        case 384: synth2<T2, 16, 16, 24>(g, f, nfield, Y, tw.th_f, s); check_launch("synth_theta"); return;
         default: break;
     }
     switch (theta_kb<T2>(g)) {
-        case 32: synth_theta_kb<T2, 32>(g, f, nfield, Y, tw_theta<T2>(tw), s); break;
-        case 16: synth_theta_kb<T2, 16>(g, f, nfield, Y, tw_theta<T2>(tw), s); break;
-        case 8: synth_theta_kb<T2, 8>(g, f, nfield, Y, tw_theta<T2>(tw), s); break;
-        default: synth_theta_kb<T2, 4>(g, f, nfield, Y, tw_theta<T2>(tw), s); break;
+        case 32: synth_theta_kb<T2, 32>(g, f, nfield, Y, tw.th_f, s); break;
+        case 16: synth_theta_kb<T2, 16>(g, f, nfield, Y, tw.th_f, s); break;
+        case 8: synth_theta_kb<T2, 8>(g, f, nfield, Y, tw.th_f, s); break;
+        default: synth_theta_kb<T2, 4>(g, f, nfield, Y, tw.th_f, s); break;
     }
     check_launch("synth_theta");
+    }
 }
 
 template <class T2>
 void launch_anal_theta(const Geo& g, const FieldPtrs& f, int nfield, const T2* Z, const Twiddles& tw, cudaStream_t s) {
+    if constexpr (std::is_same<T2, double2>::value) {
+        switch (theta_kx(g)) {
+            case 16: anal_x<16>(g, f, nfield, Z, tw.th_x, s); break;
+            case 8: anal_x<8>(g, f, nfield, Z, tw.th_x, s); break;
+            default: anal_x<4>(g, f, nfield, Z, tw.th_x, s); break;
+        }
+        check_launch("anal_theta");
+        return;
+    } else {
     switch (g.nt) {
-        case 96: anal2<T2, 32, 8, 12>(g, f, nfield, Z, tw_theta<T2>(tw), s); check_launch("anal_theta"); return;
-        case 192: anal2<T2, 32, 16, 12>(g, f, nfield, Z, tw_theta<T2>(tw), s); check_launch("anal_theta"); return;
-        case 384: anal2<T2, 16, 16, 24>(g, f, nfield, Z, tw_theta<T2>(tw), s); check_launch("anal_theta"); return;
+        case 96: anal2<T2, 32, 8, 12>(g, f, nfield, Z, tw.th_f, s); check_launch("anal_theta"); return;
+        case 192: anal2<T2, 32, 16, 12>(g, f, nfield, Z, tw.th_f, s); check_launch("anal_theta"); return;
+        case 384: anal2<T2, 16, 16, 24>(g, f, nfield, Z, tw.th_f, s); check_launch("anal_theta"); return;
         default: break;
     }
     switch (theta_kb<T2>(g)) {
-        case 32: anal_theta_kb<T2, 32>(g, f, nfield, Z, tw_theta<T2>(tw), s); break;
-        case 16: anal_theta_kb<T2, 16>(g, f, nfield, Z, tw_theta<T2>(tw), s); break;
-        case 8: anal_theta_kb<T2, 8>(g, f, nfield, Z, tw_theta<T2>(tw), s); break;
-        default: anal_theta_kb<T2, 4>(g, f, nfield, Z, tw_theta<T2>(tw), s); break;
+        case 32: anal_theta_kb<T2, 32>(g, f, nfield, Z, tw.th_f, s); break;
+        case 16: anal_theta_kb<T2, 16>(g, f, nfield, Z, tw.th_f, s); break;
+        case 8: anal_theta_kb<T2, 8>(g, f, nfield, Z, tw.th_f, s); break;
+        default: anal_theta_kb<T2, 4>(g, f, nfield, Z, tw.th_f, s); break;
     }
     check_launch("anal_theta");
+    }
 }
 
 // N/4 threads divide the radix-4 (and the radix-2, radix-3) stages of a
@@ -921,6 +1382,29 @@ static bool zpass2_any(const Geo& g, const T2* Y, T2* Z, const ZScales& sc, cons
     }
 }
 
+// FP64 forward and adjoint passes in fixed point
+template <int MODE>
+static void zpass_fixed(const Geo& g, const double2* Y, double2* Z, const ZScales& sc, const int4* tw, cudaStream_t s) {
+    constexpr int NPI = MODE == ZFWD ? 3 : 5, NG = MODE == ZFWD ? 2 : 3, NOUT = MODE == ZFWD ? 3 : 6;
+    XScales x{};
+    double gs = 1.0;
+    for (int i = 0; i < NG; ++i) {
+        int e = 0;
+        if (std::frexp(sc.hk[3 * i] / sc.h0[3 * i], &e) != 0.5 || e > 1)
+            throw std::runtime_error("zpass: unsupported input scales");
+        x.hsh[i] = 1 - e;
+        gs *= sc.h0[3 * i];  // every output is linear in each of its groups; u and w are not scaled
+    }
+    for (int i = 0; i < NOUT; ++i) {
+        x.o0[i] = sc.o0[i] * gs;
+        x.ok[i] = sc.ok[i] * gs;
+    }
+    const size_t sm = (size_t)(2 * g.nzp * NPI + g.nzp) * sizeof(double2);
+    smem_limit((const void*)k_zpass_x<MODE>);
+    launch_pdl(k_zpass_x<MODE>, dim3(g.nt, g.nr, g.nb), std::max(64u, std::min(256u, (unsigned)(g.nzp / 2 + 31) / 32 * 32)),
+               sm, s, g, Y, Z, x, tw);
+}
+
 template <class T2, int MODE>
 static void zpass_stockham(const Geo& g, const T2* Y, T2* Z, const ZScales& sc, const T2* tw, cudaStream_t s) {
     constexpr int LD = MODE == ZFWD ? 3 : (MODE == ZADJ ? 5 : 9);
@@ -941,9 +1425,12 @@ void launch_zpass(const Geo& g, int mode, const T2* Y, T2* Z, const ZScales& sc_
         sc.fok[i] = (float)sc.ok[i];
     }
     const T2* t = tw_z<T2>(tw);
-    // FP64 z passes stay on the Stockham kernel: they are bound by the FP64
-    // pipe, where the register kernel's lower occupancy measured slower.
     bool done = false;
+    if constexpr (std::is_same<T2, double2>::value) {
+        done = mode != ZCADJ;
+        if (mode == ZFWD) zpass_fixed<ZFWD>(g, Y, Z, sc, tw.z_x, s);
+        else if (mode == ZADJ) zpass_fixed<ZADJ>(g, Y, Z, sc, tw.z_x, s);
+    }
     if constexpr (std::is_same<T2, float2>::value)
         done = mode == ZFWD ? zpass2_any<T2, ZFWD>(g, Y, Z, sc, t, s)
                             : (mode == ZADJ ? zpass2_any<T2, ZADJ>(g, Y, Z, sc, t, s)
