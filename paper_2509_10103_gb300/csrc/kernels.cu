@@ -2130,7 +2130,7 @@ static void launch_band_solve(const Geo& g, const double* fac, size_t fac_stride
         }
         auto go = [&](auto kernel) {
             const dim3 grid((unsigned)((helm ? 3 : 1) * g.nm * ((g.nk + kXK - 1) / kXK)), (unsigned)gx.nb);
-            launch_serial(kernel, grid, 64, 0, s, gx, xs, fac, fac_stride, X, add, helm, zero_row0, pw, usub);
+            launch_pdl(kernel, grid, 64, 0, s, gx, xs, fac, fac_stride, X, add, helm, zero_row0, pw, usub);
         };
         if (!trans && pw) go(k_band_solve_x<false, true>);
         else if (!trans) go(k_band_solve_x<false, false>);
@@ -2176,7 +2176,7 @@ void launch_stage_finish(const Geo& g, const double2* R, const double2* addto, c
     check_launch("stage_finish");
 }
 void launch_stageT_finish(const Geo& g, const double2* ubn, double2* R, double2* ac, int ac_add, cudaStream_t s) {
-    launch_serial(k_stageT_finish, mode_grid(g), dim3(kFK, kFJ), 0, s, g, ubn, R, ac, ac_add);
+    launch_pdl(k_stageT_finish, mode_grid(g), dim3(kFK, kFJ), 0, s, g, ubn, R, ac, ac_add);
     check_launch("stageT_finish");
 }
 void launch_stageT_hsolve(const Geo& g, double2* R, const double2* add, cudaStream_t s) {
