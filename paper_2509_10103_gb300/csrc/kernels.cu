@@ -1352,8 +1352,8 @@ __global__ void k_stage_finish(Geo g, const double2* __restrict__ R, const doubl
         a0 = make_double2(p0.x + p1.x, p0.y + p1.y);
     }
     const double2 xp = R[o], xm = R[o + S];
-    double2 ur = make_double2(0.5 * (xp.x + xm.x), 0.5 * (xp.y + xm.y));
-    double2 ut = make_double2(0.5 * (xp.y - xm.y), -0.5 * (xp.x - xm.x));
+    double2 ur = make_double2(half_of(xp.x + xm.x), half_of(xp.y + xm.y));
+    double2 ut = make_double2(half_of(xp.y - xm.y), half_of(xm.x - xp.x));
     double2 uz = R[o + 2 * S];
     if (usub) {
         const double2 a = usub[o], b = usub[o + S], c = usub[o + 2 * S];
@@ -1526,8 +1526,8 @@ __global__ void __launch_bounds__(kFK* kFJ) k_stageT_finish(Geo g, const double2
         } else if (j <= 8) {
             yr = dfma(__ldg(d0 + 4 + j), acc, yr);
         }
-        R[o] = make_double2(0.5 * (yr.x - yt.y), 0.5 * (yr.y + yt.x));
-        R[o + S] = make_double2(0.5 * (yr.x + yt.y), 0.5 * (yr.y - yt.x));
+        R[o] = make_double2(half_of(yr.x - yt.y), half_of(yr.y + yt.x));
+        R[o + S] = make_double2(half_of(yr.x + yt.y), half_of(yr.y - yt.x));
         R[o + 2 * S] = yz;
     }
 }
@@ -1964,15 +1964,33 @@ __global__ void k_axpby(Geo g, size_t n, double a, const double2* __restrict__ x
     }
     out[i] = r;
 }
+// out = x + y, or (x - y) / 2 (DIFF): one FP64 instruction per part, where the
+// general form takes two and is bound by them (14.8 us at 64x64x256)
+template <bool DIFF>
+__global__ void k_sum(Geo g, size_t n, const double2* x, const double2* y, double2* out) {
+    grid_dep_sync();
+    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const size_t o = (size_t)g.slot[blockIdx.y] * g.fs + i;
+    const double2 p = x[o], q = y[o];
+    out[o] = DIFF ? make_double2(half_of(p.x - q.x), half_of(p.y - q.y)) : make_double2(p.x + q.x, p.y + q.y);
+}
 
+// x times (or over) the energy weight 2 pi Lz W_j c_k; a block covers one j,
+// whose weight one thread computes (c_k, a power of two, is an exact factor)
 __global__ void k_weight(Geo g, const double2* __restrict__ x, double2* __restrict__ out, int divide) {
     grid_dep_sync();
+    __shared__ double row;
+    if (threadIdx.x == 0) {
+        const double w = g.ewt * g.W[blockIdx.z % g.nr];
+        row = divide ? 1.0 / w : w;
+    }
+    __syncthreads();
     Idx d;
     if (!decode(g, d)) return;
     x += d.off;
     out += d.off;
-    const double w = g.ewt * g.W[d.j] * (d.k == 0 ? 1.0 : 2.0);
-    const double f = divide ? 1.0 / w : w;
+    const double f = d.k == 0 ? row : (divide ? half_of(row) : row + row);
     for (int c = 0; c < 3; ++c) {
         const size_t i = c * d.S + sidx(g, d.j, d.im, d.k);
         out[i] = make_double2(x[i].x * f, x[i].y * f);
@@ -1989,12 +2007,12 @@ __global__ void k_inner_partial(Geo g, const double2* __restrict__ a, const doub
     if (decode(g, d)) {
         a += d.off;
         b += d.off;
-        const double w = g.W[d.j] * (d.k == 0 ? 1.0 : 2.0);
         for (int c = 0; c < 3; ++c) {
             const size_t i = c * d.S + sidx(g, d.j, d.im, d.k);
             const double2 p = a[i], q = b[i];
-            acc += w * (p.x * q.x + p.y * q.y);
+            acc = fma(p.x, q.x, fma(p.y, q.y, acc));
         }
+        acc *= g.W[d.j] * (d.k == 0 ? 1.0 : 2.0);
     }
     red[threadIdx.x] = acc;
     __syncthreads();
@@ -2228,7 +2246,10 @@ void launch_project(const Geo& g, double2* u, double2* y, const double* L, cudaS
 
 void launch_axpby(const Geo& g, size_t n, double a, const double2* x, double b, const double2* y, double2* out,
                   cudaStream_t s) {
-    launch_pdl(k_axpby, dim3(nblk(n, 256), g.nb), 256, 0, s, g, n, a, x, b, y, out);
+    const dim3 grid(nblk(n, 256), g.nb);
+    if (y && a == 0.5 && b == -0.5) launch_pdl(k_sum<true>, grid, 256, 0, s, g, n, x, y, out);
+    else if (y && a == 1.0 && b == 1.0) launch_pdl(k_sum<false>, grid, 256, 0, s, g, n, x, y, out);
+    else launch_pdl(k_axpby, grid, 256, 0, s, g, n, a, x, b, y, out);
     check_launch("axpby");
 }
 void launch_weight(const Geo& g, const double2* x, double2* out, int divide, cudaStream_t s) {

@@ -1817,10 +1817,8 @@ int pnop_step_forward(pnop_ctx* ctx, void* u, double t, int nsteps) {
         ctx->pending = false;  // shares the sweep buffers
         if (!u || nsteps < 0) throw Status(PNOP_ERR_INVALID_ARG, "bad arguments");
         double2* uu = (double2*)u;
-        for (int i = 0; i < nsteps; ++i) {
-            fwd_step(ctx, uu, ctx->tmpA, t + i * ctx->h.ph.dt);
-            ck(cudaMemcpyAsync(uu, ctx->tmpA, ctx->field_bytes(), cudaMemcpyDeviceToDevice, ctx->stream), "copy");
-        }
+        // in place: the corrector, the last to write, reads only the predictor's results
+        for (int i = 0; i < nsteps; ++i) fwd_step(ctx, uu, uu, t + i * ctx->h.ph.dt);
         ck(cudaGetLastError(), "step_forward");
         return PNOP_OK;
     });
