@@ -853,7 +853,7 @@ __global__ void __launch_bounds__(2 * kSK) k_band_solve(Geo g, const double* __r
 // form 34 and 61 us: the FP64 pipe is the slower partner either way.
 constexpr int kXR = 4;         // rows per chunk
 constexpr int kXK = 16;        // systems of a block
-constexpr int kXChunks = 96;   // most chunks of a side
+constexpr int kXChunks = kFxMaxChunks;  // most chunks of a side
 struct XShape {
     int chunks[2], pad, in[2], out[2], mid[2], wall, tile;  // of FxShape
 };
@@ -2122,7 +2122,7 @@ static void launch_band_solve(const Geo& g, const double* fac, size_t fac_stride
     Geo gx = g, gd = g;
     gx.nb = gd.nb = 0;
     for (int b = 0; b < g.nb; ++b) {
-        Geo& to = (helm ? g.fxH[g.slot[b]] : g.fxP) && std::max(fx.chunks[0], fx.chunks[1]) <= kXChunks ? gx : gd;
+        Geo& to = (helm ? g.fxH[g.slot[b]] : g.fxP) ? gx : gd;
         to.slot[to.nb++] = g.slot[b];
     }
     if (gx.nb) {

@@ -630,7 +630,7 @@ static bool factor_tables(const HostOps& h, FixedTable& t, std::vector<double>& 
     const int nr = h.d.nr, nk = h.d.nk, nht = (nk + kTileX - 1) / kTileX;
     const FxShape shape = fx_shape(nr);
     auto kz = [&](int k) { return 2.0 * M_PI * k / h.d.Lz; };
-    t.ok = nr >= kFxMinRows;
+    t.ok = nr >= kFxMinRows && std::max(shape.chunks[0], shape.chunks[1]) <= kFxMaxChunks;
     t.shift = 0;
     fac.clear();
     facT.clear();

@@ -71,7 +71,8 @@ constexpr int kNc1Transposed = kUp + 1;  // A^T x = b rows: U^T (8), 1/diag | L^
 constexpr int kTileX = 16;
 constexpr int kFxBits = 58;
 constexpr double kFxRowSum = 6.0;
-constexpr int kFxMinRows = 21;  // smaller grids keep the FP64 solver
+constexpr int kFxMinRows = 21;    // smaller grids keep the FP64 solver
+constexpr int kFxMaxChunks = 96;  // chunks of a side the solver keeps units for (768 rows in all)
 struct FixedTable {
     bool ok = false;
     int shift = 0;

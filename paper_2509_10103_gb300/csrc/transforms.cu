@@ -296,7 +296,8 @@ template <int SH> __device__ __forceinline__ long long fx_dot2(xdig a, int2 c, x
     long long m = x_mad(s.y, b.l, x_mad(s.x, b.h, x_mad(c.y, a.l, x_mad(c.x, a.h, 1ll << (kXT - 33 + SH)))));
     const long long l0 = x_mul(c.x, a.l), l1 = x_mul(s.x, b.l), h = x_mad(s.y, b.h, x_mul(c.y, a.h));
     m += (long long)(int)(l0 >> 32) + (long long)(int)(l1 >> 32);
-    return (h << (64 - kXT - SH)) + (m >> (kXT - 32 + SH));
+    if (SH > 64 - kXT) return ((h << (64 - kXT - 1)) + (m >> (kXT - 31))) >> (SH - 1);
+    return (h << (64 - kXT - SH > 0 ? 64 - kXT - SH : 0)) + (m >> (kXT - 32 + SH));
 }
 // v e^{SIGN i phi} 2^-SH, w = (cos, -sin) of phi
 template <int SIGN, int SH> __device__ __forceinline__ fx2 fx_rot(fx2 v, int4 w) {
@@ -306,35 +307,58 @@ template <int SIGN, int SH> __device__ __forceinline__ fx2 fx_rot(fx2 v, int4 w)
     return SIGN < 0 ? fx2{fx_dot2<SH>(x, c, y, ns), fx_dot2<SH>(y, c, x, s)}
                     : fx2{fx_dot2<SH>(x, c, y, s), fx_dot2<SH>(y, c, x, ns)};
 }
+constexpr long long kSqrt34 = 3993837246235628775ll;  // sqrt(3)/2 2^62
+// v c, c = C 2^-kXT
+template <long long C> __device__ __forceinline__ long long fx_mul(long long v) {
+    const int2 c = make_int2((int)(unsigned)(C & 0xFFFFFFFFll), (int)((C + (1ll << 31)) >> 32));
+    return x_prod<kXT>(c, x_split(v), 1ll << (kXT - 33));
+}
+template <int SIGN> __device__ __forceinline__ fx2 fx_quarter(fx2 v) {  // SIGN i v
+    return SIGN > 0 ? fx2{-v.y, v.x} : fx2{v.y, -v.x};
+}
 template <int R, int SIGN> __device__ __forceinline__ void fx_dft(fx2* v) {
-    if (R == 2) {
+    if constexpr (R == 2) {
         const fx2 a = v[0], b = v[1];
         v[0] = fx_add(a, b);
         v[1] = fx_sub(a, b);
-    } else if (R == 4) {
-        const fx2 s02 = fx_add(v[0], v[2]), d02 = fx_sub(v[0], v[2]), s13 = fx_add(v[1], v[3]), d13 = fx_sub(v[1], v[3]);
-        const fx2 id = SIGN > 0 ? fx2{-d13.y, d13.x} : fx2{d13.y, -d13.x};
+    } else if constexpr (R == 4) {
+        const fx2 s02 = fx_add(v[0], v[2]), d02 = fx_sub(v[0], v[2]), s13 = fx_add(v[1], v[3]);
+        const fx2 id = fx_quarter<SIGN>(fx_sub(v[1], v[3]));
         v[0] = fx_add(s02, s13);
         v[2] = fx_sub(s02, s13);
         v[1] = fx_add(d02, id);
         v[3] = fx_sub(d02, id);
+    } else if constexpr (R == 6) {  // n = 3 a + 2 b, k = 3 (k mod 2) + 4 (k mod 3) mod 6: no turns in between
+        fx2 t[2][3];
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const fx2 p = v[(2 * b) % 6], q = v[(3 + 2 * b) % 6];
+            t[0][b] = fx_add(p, q);
+            t[1][b] = fx_sub(p, q);
+        }
+        fx_dft<3, SIGN>(t[0]);
+        fx_dft<3, SIGN>(t[1]);
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            v[(4 * b) % 6] = t[0][b];
+            v[(3 + 4 * b) % 6] = t[1][b];
+        }
     } else {  // R == 3
-        constexpr long long h = 3993837246235628775ll;  // sqrt(3)/2 2^62
-        const int2 hd = make_int2((int)(unsigned)(h & 0xFFFFFFFFll), (int)((h + (1ll << 31)) >> 32));
         const fx2 t1 = fx_add(v[1], v[2]), d = fx_sub(v[1], v[2]);
         const fx2 t2 = {v[0].x - (t1.x >> 1), v[0].y - (t1.y >> 1)};
-        const long long px = x_prod<kXT>(hd, x_split(d.x), 1ll << (kXT - 33)), py = x_prod<kXT>(hd, x_split(d.y), 1ll << (kXT - 33));
-        const fx2 t3 = SIGN > 0 ? fx2{-py, px} : fx2{py, -px};
+        const fx2 t3 = fx_quarter<SIGN>(fx2{fx_mul<kSqrt34>(d.x), fx_mul<kSqrt34>(d.y)});
         v[0] = fx_add(v[0], t1);
         v[1] = fx_add(t2, t3);
         v[2] = fx_sub(t2, t3);
     }
 }
+// bits a radix-R stage can grow by
+__host__ __device__ constexpr int fx_growth(int R) { return R == 2 ? 1 : (R <= 4 ? 2 : 3); }
 // the Stockham stages of fft_cols in fixed point
 template <int R, int NCOL, int LD, int SIGN, bool SCALE>
 __device__ __forceinline__ void fx_stage(const fx2* __restrict__ a, fx2* __restrict__ b, int N, int Ns, int lgNs,
                                          const int4* __restrict__ tw) {
-    constexpr int SH = !SCALE ? 0 : (R == 2 ? 1 : 2);  // what the stage can grow by (the first stage is not scaled)
+    constexpr int SH = !SCALE ? 0 : fx_growth(R);  // the first stage is not scaled
     const int stride = N / R, nb = stride * NCOL, tstep = N / (Ns * R);
     for (int idx = threadIdx.x; idx < nb; idx += blockDim.x) {
         const int col = idx % NCOL, jb = idx / NCOL;
@@ -353,7 +377,7 @@ __device__ __forceinline__ void fx_stage(const fx2* __restrict__ a, fx2* __restr
             const int tb = kk * tstep;
 #pragma unroll
             for (int r = 1; r < R; ++r) v[r] = fx_rot<SIGN, SH>(v[r], tw[r * tb]);
-            if (SCALE) v[0] = {(v[0].x + SH) >> SH, (v[0].y + SH) >> SH};  // SH = 1 or 2: half a unit is SH
+            if (SCALE) v[0] = {(v[0].x + (1ll << SH >> 1)) >> SH, (v[0].y + (1ll << SH >> 1)) >> SH};
         }
         fx_dft<R, SIGN>(v);
         const int idxD = q * Ns * R + kk;
@@ -364,8 +388,7 @@ __device__ __forceinline__ void fx_stage(const fx2* __restrict__ a, fx2* __restr
 // halvings: what the result is to be multiplied by, as an exponent of 2 (SCALE)
 template <int NCOL, int LD, int SIGN, bool SCALE = false>
 __device__ fx2* fx_cols(fx2* a, fx2* b, int N, const int4* tw, int* halvings = nullptr) {
-    const int n2 = __ffs(N) - 1;
-    int n3 = 0;
+    int n2 = __ffs(N) - 1, n3 = 0;
     for (int t = N >> n2; t > 1; t /= 3) ++n3;
     int Ns = 1, lgNs = 0;
     auto next = [&](int R) {
@@ -373,22 +396,30 @@ __device__ fx2* fx_cols(fx2* a, fx2* b, int N, const int4* tw, int* halvings = n
         fx2* t = a;
         a = b;
         b = t;
-        if (SCALE && Ns > 1) *halvings += R == 2 ? 1 : 2;
+        if (SCALE && Ns > 1) *halvings += fx_growth(R);
         Ns *= R;
     };
-    for (int st = 0; st < n2 / 2; ++st) {
+    // radix 4, a remaining 2 with a 3 as radix 6 (64x64x256 z pass: 197 and 358 us;
+    // with radix 2 and 3 apart 215 and 387, with radix 8 and 6 227 and 350)
+    for (; n2 >= 2; n2 -= 2) {
         fx_stage<4, NCOL, LD, SIGN, SCALE>(a, b, N, Ns, lgNs, tw);
         next(4);
         lgNs += 2;
     }
-    if (n2 & 1) {
+    if (n2 == 1 && n3 > 0) {
+        fx_stage<6, NCOL, LD, SIGN, SCALE>(a, b, N, Ns, lgNs, tw);
+        next(6);
+        lgNs = -1;
+        --n3;
+    } else if (n2 == 1) {
         fx_stage<2, NCOL, LD, SIGN, SCALE>(a, b, N, Ns, lgNs, tw);
         next(2);
         lgNs += 1;
     }
-    for (int st = 0; st < n3; ++st) {
-        fx_stage<3, NCOL, LD, SIGN, SCALE>(a, b, N, Ns, st == 0 ? lgNs : -1, tw);
+    for (; n3 > 0; --n3) {
+        fx_stage<3, NCOL, LD, SIGN, SCALE>(a, b, N, Ns, lgNs, tw);
         next(3);
+        lgNs = -1;
     }
     return a;
 }
@@ -405,7 +436,10 @@ __device__ __forceinline__ int fx_unit(unsigned sum, int top, int bits) {
 }
 __device__ __forceinline__ int x_top(long long v) { return 64 - __clzll(v ^ (v >> 63)); }  // |v| <= 2^top
 
-// the z pass in fixed point: contract of k_zpass (FP64), any length.  The fields
+// The z pass in fixed point: contract of k_zpass (FP64), any length.  Bound by
+// integer issue and its barriers (44% of the warps' slots in use at 64x64x256);
+// 828 -> 197 us forward and 1308 -> 358 us adjoint against the FP64 Stockham
+// kernel, 73 and 108 FP64 instructions a point at 77 cycles.  The fields
 // fall into the groups u, w and (modes ZADJ, ZCADJ) g, each with one unit; a
 // group's input scale is gs for k = 0 and gs hs for k > 0, hs a power of two (hsh
 // its exponent), and gs is part of the output scales o0, ok.
@@ -429,6 +463,7 @@ __global__ void k_zpass_x(Geo g, const double2* __restrict__ Y, double2* __restr
     fx2* bufA = reinterpret_cast<fx2*>(smem);
     fx2* bufB = bufA + N * NPI;
     int4* tw = reinterpret_cast<int4*>(bufB + N * NPI);
+    auto at = [](int n, int p) { return n * NPI + p; };
     const int a = blockIdx.x, j = blockIdx.y;
     const size_t poff = (size_t)g.slot[blockIdx.z] * g.ps;
     Y += poff;
@@ -479,7 +514,7 @@ __global__ void k_zpass_x(Geo g, const double2* __restrict__ Y, double2* __restr
     for (int i = 0; i < NG; ++i)
         E[i] = max(fx_unit(max(sum_sh[3 * i], max(sum_sh[3 * i + 1], sum_sh[3 * i + 2])), top[i], 59), -kXTop);
     // Hermitian-extended spectra, two fields per column
-    for (int n = threadIdx.x; n < NPI * (N - 2 * nk + 1); n += blockDim.x) bufA[nk * NPI + n] = {0, 0};
+    for (int n = threadIdx.x; n < NPI * (N - 2 * nk + 1); n += blockDim.x) bufA[at(nk, n)] = {0, 0};
 #pragma unroll
     for (int p = 0; p < NPI; ++p) {
         constexpr int none = NIN;
@@ -493,8 +528,8 @@ __global__ void k_zpass_x(Geo g, const double2* __restrict__ Y, double2* __restr
                 h1 = {h1.x >> sc.hsh[g1], h1.y >> sc.hsh[g1]};
                 h2 = {h2.x >> sc.hsh[g2], h2.y >> sc.hsh[g2]};
             }
-            bufA[k * NPI + p] = {h1.x - h2.y, h1.y + h2.x};                    // H1 + i H2
-            if (k > 0) bufA[(N - k) * NPI + p] = {h1.x + h2.y, h2.x - h1.y};  // conj(H1) + i conj(H2)
+            bufA[at(k, p)] = {h1.x - h2.y, h1.y + h2.x};                    // H1 + i H2
+            if (k > 0) bufA[at(N - k, p)] = {h1.x + h2.y, h2.x - h1.y};  // conj(H1) + i conj(H2)
         }
     }
     __syncthreads();
@@ -504,9 +539,12 @@ __global__ void k_zpass_x(Geo g, const double2* __restrict__ Y, double2* __restr
     {
         long long mx[3] = {};
         for (int n = threadIdx.x; n < N; n += blockDim.x) {
-            const long long* row = reinterpret_cast<const long long*>(ph + n * NPI);
 #pragma unroll
-            for (int f = 0; f < NIN; ++f) mx[f / 3] |= row[f] ^ (row[f] >> 63);
+            for (int f = 0; f < NIN; ++f) {
+                const fx2 c = ph[at(n, f / 2)];
+                const long long x = f % 2 ? c.y : c.x;
+                mx[f / 3] |= x ^ (x >> 63);
+            }
         }
 #pragma unroll
         for (int i = 0; i < NG; ++i) {
@@ -516,8 +554,10 @@ __global__ void k_zpass_x(Geo g, const double2* __restrict__ Y, double2* __restr
     }
     __syncthreads();
     // a product (a b - c d) is shifted by 60 + sh, so that two of them stay below
-    // 2^59 (the first stage of the forward transform at most quadruples them)
-    auto shift = [&](int ga, int gb) { return max(max_sh[ga] + max_sh[gb] + 2 - 60 - 59, 0); };
+    // 2^61 over what the first stage of the forward transform adds up: four, or
+    // where N is not a multiple of four up to six
+    const int room = N % 4 == 0 ? 59 : 58;
+    auto shift = [&](int ga, int gb) { return max(max_sh[ga] + max_sh[gb] + 2 - 60 - room, 0); };
     auto cross = [&](xdig p, xdig q, xdig nr, xdig t, int sh) {  // (p q + nr t) >> (60 + sh)
         long long m = x_mad(nr.h, t.l, x_mad(nr.l, t.h, x_mad(p.h, q.l, x_mul(p.l, q.h))));
         const long long l0 = x_mul(p.l, q.l), l1 = x_mul(nr.l, t.l), h = x_mad(nr.h, t.h, x_mul(p.h, q.h));
@@ -526,14 +566,20 @@ __global__ void k_zpass_x(Geo g, const double2* __restrict__ Y, double2* __restr
     };
     const int s01 = shift(0, 1), s12 = MODE == ZADJ ? shift(1, 2) : 0, s02 = MODE == ZADJ ? shift(0, 2) : 0;
     for (int n = threadIdx.x; n < N; n += blockDim.x) {
-        const long long* row = reinterpret_cast<const long long*>(ph + n * NPI);
+        long long row[2 * NPI];
+#pragma unroll
+        for (int p = 0; p < NPI; ++p) {
+            const fx2 c = ph[at(n, p)];
+            row[2 * p] = c.x;
+            row[2 * p + 1] = c.y;
+        }
         xdig v[NIN], n_[NIN];  // digits of the values and of their negatives
 #pragma unroll
         for (int f = 0; f < NIN; ++f) {
             v[f] = x_split(row[f]);
             n_[f] = x_split(-row[f]);
         }
-        fx2* o = pr + n * NPI;
+        fx2 o[3];
         if (MODE == ZFWD) {  // u x w
             o[0] = {cross(v[1], v[5], n_[2], v[4], s01), cross(v[2], v[3], n_[0], v[5], s01)};
             o[1] = {cross(v[0], v[4], n_[1], v[3], s01), 0};
@@ -543,6 +589,8 @@ __global__ void k_zpass_x(Geo g, const double2* __restrict__ Y, double2* __restr
             o[1] = {cross(v[3], v[g0 + 1], n_[4], v[g0], s12), cross(v[g0 + 1], v[2], n_[1], v[g0 + 2], s02)};
             o[2] = {cross(v[g0 + 2], v[0], n_[2], v[g0], s02), cross(v[g0], v[1], n_[0], v[g0 + 1], s02)};
         }
+#pragma unroll
+        for (int p = 0; p < NPO; ++p) pr[at(n, p)] = o[p];
     }
     __syncthreads();
     int halvings = 0;
@@ -563,14 +611,15 @@ __global__ void k_zpass_x(Geo g, const double2* __restrict__ Y, double2* __restr
 #pragma unroll
     for (int p = 0; p < NPO; ++p)
         for (int k = threadIdx.x; k < nk; k += blockDim.x) {
-            const fx2 P = sp[k * NPI + p], Q = sp[(k ? N - k : 0) * NPI + p];
+            const fx2 P = sp[at(k, p)], Q = sp[at(k ? N - k : 0, p)];
             put(2 * p, k, P.x + Q.x, P.y - Q.y);
             if (2 * p + 1 < NOUT) put(2 * p + 1, k, P.y + Q.y, Q.x - P.x);
         }
 }
 
 // The theta transforms in fixed point, any length: contract of k_synth_theta and
-// k_anal_theta (FP64).  A block takes KB columns k of one (field, j), all in one
+// k_anal_theta (FP64).  206 -> 74 us (synthesis) and 158 -> 64 us (analysis) at
+// 64x64x256 against the FP64 two-pass kernels.  A block takes KB columns k of one (field, j), all in one
 // unit (the z pass sums over k, so a column far below its neighbours does not
 // count there).  Rows of `in` values from memory into `raw`, and the unit in
 // which the magnitudes of every column sum to less than 2^61; bad: infinities or NaN.
