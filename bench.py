@@ -106,10 +106,11 @@ def class_work(cls, units, mixed):
     return None, None
 
 
-KERNEL_SOURCES = ("kernels.cu", "transforms.cu", "kernels.hpp", "dev_common.cuh", "dev_df.cuh")
+KERNEL_SOURCES = ("kernels.cu", "transforms.cu", "kernels.hpp", "dev_common.cuh", "dev_df.cuh", "dev_x64.cuh")
 # the translation unit and headers that define a class's kernels: the banded
-# solves live in kernels.cu, which the transforms' unit cannot change
-CLASS_SOURCES = {"radial_solve": ("kernels.cu", "kernels.hpp", "dev_common.cuh", "dev_df.cuh")}
+# solves and products live in kernels.cu, which the transforms' unit cannot change
+CLASS_SOURCES = dict.fromkeys(("radial_solve", "radial_band"),
+                              ("kernels.cu", "kernels.hpp", "dev_common.cuh", "dev_df.cuh", "dev_x64.cuh"))
 
 
 def kernel_digest(cls=None):
