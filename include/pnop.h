@@ -61,8 +61,7 @@ enum {
  *   PNOP_DF (2): the explicit banded radial products (curl, divergence,
  *     pressure gradient and their transposes) in double-FP32 arithmetic
  *     (about 48 significant bits, Dekker 1971), since FP64 runs at 1/64 of
- *     the FP32 rate on this GPU.  (With PNOP_MIXED alone, so do the curl and
- *     its transpose, whose vorticity is an FP32 field then.)
+ *     the FP32 rate on this GPU.
  * Everything else (the radial banded solves, the influence and flux
  * corrections, the base flow, the stage combinations, energies and inner
  * products) stays FP64.  PNOP_FP64 (0) is FP64 throughout.  In every precision

@@ -1713,7 +1713,7 @@ int create_impl(const pnop_grid* grid, const pnop_params* params, void* cuda_str
             g.kzt = c->upload(kz);
             g.mrt = c->upload(mr);
             g.df = (params->precision & PNOP_DF) ? 1 : 0;
-            if (params->precision != PNOP_FP64) {  // FP32 vorticity takes the double-FP32 curl too
+            if (g.df) {
                 g.D1f = c->upload(split_pairs(c->h.D1));
                 g.invrf = c->upload(split_pairs(c->h.invr));
                 g.kztf = c->upload(split_pairs(kz));
