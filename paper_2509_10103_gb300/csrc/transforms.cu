@@ -283,8 +283,9 @@ __global__ void k_zpass(Geo g, const T2* __restrict__ Y, T2* __restrict__ Z, ZSc
 // transform share one exponent.  For spectra it is chosen from the sum of the
 // magnitudes of the inputs, which bounds every intermediate result: a unit is
 // 2^-60 of that sum.  The forward z transform takes its values, products of
-// physical fields, at full length and halves them as often as a stage can double
-// them (SCALE).  Nothing can wrap either way.
+// physical fields, at full length (the largest below 2^58, moved there in the
+// first stage) and divides them by the power of two that the stages so far can
+// have multiplied them by (SCALE).  Nothing can wrap either way.
 struct fx2 {
     long long x, y;
 };
@@ -352,13 +353,23 @@ template <int R, int SIGN> __device__ __forceinline__ void fx_dft(fx2* v) {
         v[2] = fx_sub(t2, t3);
     }
 }
-// bits a radix-R stage can grow by
-__host__ __device__ constexpr int fx_growth(int R) { return R == 2 ? 1 : (R <= 4 ? 2 : 3); }
-// the Stockham stages of fft_cols in fixed point
-template <int R, int NCOL, int LD, int SIGN, bool SCALE>
+// bits that n values of a sum can add
+__host__ __device__ constexpr int fx_growth(int n) {
+    int b = 0;
+    while ((1 << b) < n) ++b;
+    return b;
+}
+// Bits by which the first stage moves up the real (i = 0) and imaginary part of
+// column col, so that the largest value fills `room` bits.
+struct xlift {
+    const int* top;  // bits of the largest values of the columns' parts
+    int room;
+    __device__ __forceinline__ int operator()(int col, int i) const { return max(room - top[2 * col + i], 0); }
+};
+// the Stockham stages of fft_cols in fixed point, scaled by 2^-SH
+template <int R, int NCOL, int LD, int SIGN, int SH>
 __device__ __forceinline__ void fx_stage(const fx2* __restrict__ a, fx2* __restrict__ b, int N, int Ns, int lgNs,
-                                         const int4* __restrict__ tw) {
-    constexpr int SH = !SCALE ? 0 : fx_growth(R);  // the first stage is not scaled
+                                         const int4* __restrict__ tw, const xlift* lift) {
     const int stride = N / R, nb = stride * NCOL, tstep = N / (Ns * R);
     for (int idx = threadIdx.x; idx < nb; idx += blockDim.x) {
         const int col = idx % NCOL, jb = idx / NCOL;
@@ -373,11 +384,16 @@ __device__ __forceinline__ void fx_stage(const fx2* __restrict__ a, fx2* __restr
         fx2 v[R];
 #pragma unroll
         for (int r = 0; r < R; ++r) v[r] = a[(jb + r * stride) * LD + col];
+        if (lift) {
+            const int lx = (*lift)(col, 0), ly = (*lift)(col, 1);
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[r] = {v[r].x << lx, v[r].y << ly};
+        }
         if (Ns > 1) {
             const int tb = kk * tstep;
 #pragma unroll
             for (int r = 1; r < R; ++r) v[r] = fx_rot<SIGN, SH>(v[r], tw[r * tb]);
-            if (SCALE) v[0] = {(v[0].x + (1ll << SH >> 1)) >> SH, (v[0].y + (1ll << SH >> 1)) >> SH};
+            if (SH) v[0] = {(v[0].x + (1ll << SH >> 1)) >> SH, (v[0].y + (1ll << SH >> 1)) >> SH};
         }
         fx_dft<R, SIGN>(v);
         const int idxD = q * Ns * R + kk;
@@ -385,40 +401,47 @@ __device__ __forceinline__ void fx_stage(const fx2* __restrict__ a, fx2* __restr
         for (int r = 0; r < R; ++r) b[(idxD + r * Ns) * LD + col] = v[r];
     }
 }
-// halvings: what the result is to be multiplied by, as an exponent of 2 (SCALE)
+// halvings: what the result is to be multiplied by, as an exponent of 2 (SCALE).
+// The first stage is not scaled; after it a value is at most 2^fx_growth(first
+// radix) times the largest input, and stays so.
 template <int NCOL, int LD, int SIGN, bool SCALE = false>
-__device__ fx2* fx_cols(fx2* a, fx2* b, int N, const int4* tw, int* halvings = nullptr) {
+__device__ fx2* fx_cols(fx2* a, fx2* b, int N, const int4* tw, int* halvings = nullptr, const xlift* lift = nullptr) {
     int n2 = __ffs(N) - 1, n3 = 0;
     for (int t = N >> n2; t > 1; t /= 3) ++n3;
     int Ns = 1, lgNs = 0;
-    auto next = [&](int R) {
+    auto next = [&](int R, int SH) {
         __syncthreads();
         fx2* t = a;
         a = b;
         b = t;
-        if (SCALE && Ns > 1) *halvings += fx_growth(R);
+        if (SCALE && Ns > 1) *halvings += SH;
         Ns *= R;
+        lift = nullptr;
     };
-    // radix 4, a remaining 2 with a 3 as radix 6 (64x64x256 z pass: 197 and 358 us;
-    // with radix 2 and 3 apart 215 and 387, with radix 8 and 6 227 and 350)
+    // radix 4, a remaining 2 with a 3 as radix 6 (64x64x256 z pass, before its fields
+    // had units of their own: 197 and 358 us; with radix 2 and 3 apart 215 and 387,
+    // with radix 8 and 6 227 and 350).  Radix 4, 2 and 6 follow powers of four, so that
+    // a stage's scale depends on the radix alone; radix 3 takes one or two bits (3, 9, 27, 81, 243 times: 2, 4, 5, 7, 8).
     for (; n2 >= 2; n2 -= 2) {
-        fx_stage<4, NCOL, LD, SIGN, SCALE>(a, b, N, Ns, lgNs, tw);
-        next(4);
+        fx_stage<4, NCOL, LD, SIGN, SCALE ? 2 : 0>(a, b, N, Ns, lgNs, tw, lift);
+        next(4, 2);
         lgNs += 2;
     }
     if (n2 == 1 && n3 > 0) {
-        fx_stage<6, NCOL, LD, SIGN, SCALE>(a, b, N, Ns, lgNs, tw);
-        next(6);
+        fx_stage<6, NCOL, LD, SIGN, SCALE ? 3 : 0>(a, b, N, Ns, lgNs, tw, lift);
+        next(6, 3);
         lgNs = -1;
         --n3;
     } else if (n2 == 1) {
-        fx_stage<2, NCOL, LD, SIGN, SCALE>(a, b, N, Ns, lgNs, tw);
-        next(2);
+        fx_stage<2, NCOL, LD, SIGN, SCALE ? 1 : 0>(a, b, N, Ns, lgNs, tw, lift);
+        next(2, 1);
         lgNs += 1;
     }
     for (; n3 > 0; --n3) {
-        fx_stage<3, NCOL, LD, SIGN, SCALE>(a, b, N, Ns, lgNs, tw);
-        next(3);
+        const bool two = SCALE && fx_growth(3 * Ns) - fx_growth(Ns) == 2;
+        if (two) fx_stage<3, NCOL, LD, SIGN, SCALE ? 2 : 0>(a, b, N, Ns, lgNs, tw, lift);
+        else fx_stage<3, NCOL, LD, SIGN, SCALE ? 1 : 0>(a, b, N, Ns, lgNs, tw, lift);
+        next(3, two ? 2 : 1);
         lgNs = -1;
     }
     return a;
@@ -438,26 +461,36 @@ __device__ __forceinline__ int x_top(long long v) { return 64 - __clzll(v ^ (v >
 
 // The z pass in fixed point: contract of k_zpass (FP64), any length.  Bound by
 // integer issue and its barriers (44% of the warps' slots in use at 64x64x256);
-// 828 -> 197 us forward and 1308 -> 358 us adjoint against the FP64 Stockham
-// kernel, 73 and 108 FP64 instructions a point at 77 cycles.  The fields
-// fall into the groups u, w and (modes ZADJ, ZCADJ) g, each with one unit; a
-// group's input scale is gs for k = 0 and gs hs for k > 0, hs a power of two (hsh
-// its exponent), and gs is part of the output scales o0, ok.
+// 828 -> 207 us forward and 1308 -> 334 us adjoint against the FP64 Stockham
+// kernel, 73 and 108 FP64 instructions a point at 77 cycles.  Every field has a
+// unit of its own (the components of u and of w differ by orders of magnitude
+// in streaky flows), and every output one from the larger of its two products:
+// a component's error is 1.0e-16 to 2.3e-16 of its root mean square at 24 to 243
+// points (FP64 arithmetic: 2e-16 to 6e-16, and up to 2e-12 where a small
+// component shared a packed column with a large one).  At most 80 registers:
+// 43.6 -> 41.9 us at 48x32x96, whose blocks are the smaller for it.
+// The fields fall into the groups u, w and (mode ZADJ) g; a group's input scale
+// is gs for k = 0 and gs hs for k > 0, hs a power of two (hsh its exponent),
+// and gs is part of the output scales o0, ok.
 struct XScales {
     int hsh[3];
     double o0[6], ok[6];
 };
+constexpr int kXProd = 59;  // a product of two fields, each below 2^60, keeps its bits from here on
+__device__ __forceinline__ long long fx_prod(xdig p, xdig q) {
+    const long long m = x_mad(p.h, q.l, x_mul(p.l, q.h)) + (long long)(int)(x_mul(p.l, q.l) >> 32);
+    return (x_mul(p.h, q.h) << (64 - kXProd)) + (m >> (kXProd - 32));
+}
 template <int MODE>
-__global__ void k_zpass_x(Geo g, const double2* __restrict__ Y, double2* __restrict__ Z, XScales sc,
-                          const int4* __restrict__ twg) {
+__global__ void __launch_bounds__(256, 3)
+    k_zpass_x(Geo g, const double2* __restrict__ Y, double2* __restrict__ Z, XScales sc, const int4* __restrict__ twg) {
     grid_dep_sync();
     constexpr int NIN = MODE == ZFWD ? 6 : 9;
     constexpr int NPI = (NIN + 1) / 2;
     constexpr int NOUT = MODE == ZADJ ? 6 : 3;
     constexpr int NPO = (NOUT + 1) / 2;
-    constexpr int NG = NIN / 3;
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int top_sh[3], max_sh[3];
+    __shared__ int top_sh[NIN], max_sh[NIN], out_sh[NOUT][3], omax_sh[2 * NPO];
     __shared__ unsigned sum_sh[NIN];
     const int N = g.nzp, nk = g.nk;
     fx2* bufA = reinterpret_cast<fx2*>(smem);
@@ -468,66 +501,72 @@ __global__ void k_zpass_x(Geo g, const double2* __restrict__ Y, double2* __restr
     const size_t poff = (size_t)g.slot[blockIdx.z] * g.ps;
     Y += poff;
     Z += poff;
-    if (threadIdx.x < 3) top_sh[threadIdx.x] = max_sh[threadIdx.x] = 0;
-    if (threadIdx.x < NIN) sum_sh[threadIdx.x] = 0;
+    if (threadIdx.x < NIN) top_sh[threadIdx.x] = max_sh[threadIdx.x] = sum_sh[threadIdx.x] = 0;
+    if (threadIdx.x < 2 * NPO) omax_sh[threadIdx.x] = 0;
     for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = twg[i];
     __syncthreads();
-    // inputs into bufB as they are, the largest exponent of each group
+    // inputs into bufB as they are, the largest exponent of each field
     double2* raw = reinterpret_cast<double2*>(bufB);  // [NIN][nk]
     {
-        int mx[NG] = {};
+        int mx[NIN] = {};
+        for (int k = threadIdx.x; k < nk; k += blockDim.x) {
+            double2 y[NIN];
 #pragma unroll
-        for (int f = 0; f < NIN; ++f)
-            for (int k = threadIdx.x; k < nk; k += blockDim.x) {
-                double2 y = Y[((size_t)(f * g.nr + j) * g.nt + a) * nk + k];
-                if (k == 0) y.y = 0;
-                raw[f * nk + k] = y;
-                mx[f / 3] = max(mx[f / 3], max(__double2hiint(y.x) & 0x7FFFFFFF, __double2hiint(y.y) & 0x7FFFFFFF));
+            for (int f = 0; f < NIN; ++f) y[f] = Y[((size_t)(f * g.nr + j) * g.nt + a) * nk + k];
+#pragma unroll
+            for (int f = 0; f < NIN; ++f) {
+                if (k == 0) y[f].y = 0;
+                raw[f * nk + k] = y[f];
+                mx[f] = max(mx[f], max(__double2hiint(y[f].x) & 0x7FFFFFFF, __double2hiint(y[f].y) & 0x7FFFFFFF));
             }
-#pragma unroll
-        for (int i = 0; i < NG; ++i) {
-            const int m = __reduce_max_sync(0xffffffffu, mx[i]);
-            if ((threadIdx.x & 31) == 0) atomicMax(&top_sh[i], m);
         }
+#pragma unroll
+        for (int f = 0; f < NIN; ++f) mx[f] = __reduce_max_sync(0xffffffffu, mx[f]);
+        if ((threadIdx.x & 31) == 0)
+#pragma unroll
+            for (int f = 0; f < NIN; ++f) atomicMax(&top_sh[f], mx[f]);
     }
     __syncthreads();
     bool bad = false;
-    int top[NG];
+    {
+        unsigned sum[NIN] = {};
+        int top[NIN];
 #pragma unroll
-    for (int i = 0; i < NG; ++i) {
-        bad = bad || top_sh[i] >= 0x7FF00000;
-        top[i] = top_sh[i] >> 20;
-    }
-#pragma unroll
-    for (int f = 0; f < NIN; ++f) {
-        unsigned s = 0;
-        for (int k = threadIdx.x; k < nk; k += blockDim.x) {
-            const double2 y = raw[f * nk + k];
-            s += (fx_count(y.x, top[f / 3]) + fx_count(y.y, top[f / 3]) + 3u) >> 2;  // nk up to 2^12
+        for (int f = 0; f < NIN; ++f) {
+            bad = bad || top_sh[f] >= 0x7FF00000;
+            top[f] = top_sh[f] >> 20;
         }
-        s = __reduce_add_sync(0xffffffffu, s);
-        if ((threadIdx.x & 31) == 0) atomicAdd(&sum_sh[f], s);
+        for (int k = threadIdx.x; k < nk; k += blockDim.x) {
+#pragma unroll
+            for (int f = 0; f < NIN; ++f) {
+                const double2 y = raw[f * nk + k];
+                sum[f] += (fx_count(y.x, top[f]) + fx_count(y.y, top[f]) + 3u) >> 2;  // nk up to 2^12
+            }
+        }
+#pragma unroll
+        for (int f = 0; f < NIN; ++f) sum[f] = __reduce_add_sync(0xffffffffu, sum[f]);
+        if ((threadIdx.x & 31) == 0)
+#pragma unroll
+            for (int f = 0; f < NIN; ++f) atomicAdd(&sum_sh[f], sum[f]);
     }
     __syncthreads();
-    int E[NG];  // |f| <= 2 sum of the magnitudes < 2^60 units; a packed column < 2^61
-#pragma unroll
-    for (int i = 0; i < NG; ++i)
-        E[i] = max(fx_unit(max(sum_sh[3 * i], max(sum_sh[3 * i + 1], sum_sh[3 * i + 2])), top[i], 59), -kXTop);
+    // |f| <= 2 sum of the magnitudes < 2^60 units; a packed column < 2^61
+    auto unit = [&](int f) { return max(fx_unit(sum_sh[f], top_sh[f] >> 20, 59), -kXTop); };
     // Hermitian-extended spectra, two fields per column
     for (int n = threadIdx.x; n < NPI * (N - 2 * nk + 1); n += blockDim.x) bufA[at(nk, n)] = {0, 0};
 #pragma unroll
     for (int p = 0; p < NPI; ++p) {
         constexpr int none = NIN;
         const int f1 = 2 * p, f2 = 2 * p + 1 < NIN ? 2 * p + 1 : none, g1 = f1 / 3, g2 = f2 == none ? g1 : f2 / 3;
-        const xunit u1 = x_unit(E[g1]), u2 = x_unit(E[g2]);
+        const int e1 = unit(f1), e2 = f2 == none ? e1 : unit(f2);
+        const xunit u01 = x_unit(e1), u02 = x_unit(e2);  // k = 0
+        const xunit u1 = MODE == ZADJ ? x_unit(e1 + sc.hsh[g1]) : u01, u2 = MODE == ZADJ ? x_unit(e2 + sc.hsh[g2]) : u02;
         for (int k = threadIdx.x; k < nk; k += blockDim.x) {
             const double2 y1 = raw[f1 * nk + k], y2 = f2 == none ? make_double2(0, 0) : raw[f2 * nk + k];
-            fx2 h1 = {x_load(y1.x, u1), x_load(y1.y, u1)}, h2 = {0, 0};
-            if (f2 != none) h2 = {x_load(y2.x, u2), x_load(y2.y, u2)};
-            if (k > 0 && MODE == ZADJ) {
-                h1 = {h1.x >> sc.hsh[g1], h1.y >> sc.hsh[g1]};
-                h2 = {h2.x >> sc.hsh[g2], h2.y >> sc.hsh[g2]};
-            }
+            const xunit v1 = k ? u1 : u01, v2 = k ? u2 : u02;
+            const fx2 h1 = {x_load(y1.x, v1), x_load(y1.y, v1)};
+            fx2 h2 = {0, 0};
+            if (f2 != none) h2 = {x_load(y2.x, v2), x_load(y2.y, v2)};
             bufA[at(k, p)] = {h1.x - h2.y, h1.y + h2.x};                    // H1 + i H2
             if (k > 0) bufA[at(N - k, p)] = {h1.x + h2.y, h2.x - h1.y};  // conj(H1) + i conj(H2)
         }
@@ -535,73 +574,100 @@ __global__ void k_zpass_x(Geo g, const double2* __restrict__ Y, double2* __restr
     __syncthreads();
     fx2* ph = fx_cols<NPI, NPI, +1>(bufA, bufB, N, tw);
     fx2* pr = ph == bufA ? bufB : bufA;
-    // largest physical values of the groups, for the units of the products
+    // largest physical values of the fields, for the units of the products
     {
-        long long mx[3] = {};
+        long long mx[NIN] = {};
         for (int n = threadIdx.x; n < N; n += blockDim.x) {
 #pragma unroll
             for (int f = 0; f < NIN; ++f) {
                 const fx2 c = ph[at(n, f / 2)];
                 const long long x = f % 2 ? c.y : c.x;
-                mx[f / 3] |= x ^ (x >> 63);
+                mx[f] |= x ^ (x >> 63);
             }
         }
+        int m[NIN];
 #pragma unroll
-        for (int i = 0; i < NG; ++i) {
-            const int m = __reduce_max_sync(0xffffffffu, x_top(mx[i]));
-            if ((threadIdx.x & 31) == 0) atomicMax(&max_sh[i], m);
-        }
+        for (int f = 0; f < NIN; ++f) m[f] = __reduce_max_sync(0xffffffffu, x_top(mx[f]));
+        if ((threadIdx.x & 31) == 0)
+#pragma unroll
+            for (int f = 0; f < NIN; ++f) atomicMax(&max_sh[f], m[f]);
     }
     __syncthreads();
-    // a product (a b - c d) is shifted by 60 + sh, so that two of them stay below
-    // 2^61 over what the first stage of the forward transform adds up: four, or
-    // where N is not a multiple of four up to six
-    const int room = N % 4 == 0 ? 59 : 58;
-    auto shift = [&](int ga, int gb) { return max(max_sh[ga] + max_sh[gb] + 2 - 60 - room, 0); };
-    auto cross = [&](xdig p, xdig q, xdig nr, xdig t, int sh) {  // (p q + nr t) >> (60 + sh)
-        long long m = x_mad(nr.h, t.l, x_mad(nr.l, t.h, x_mad(p.h, q.l, x_mul(p.l, q.h))));
-        const long long l0 = x_mul(p.l, q.l), l1 = x_mul(nr.l, t.l), h = x_mad(nr.h, t.h, x_mul(p.h, q.h));
-        m += (long long)(int)(l0 >> 32) + (long long)(int)(l1 >> 32);
-        return ((h << 4) + (m >> 28)) >> sh;
+    // Output f = p q - r t: (w x g) for the adjoint pass, then u x w or g x u.
+    // The fields are moved up to 2^60 first, so that the products take shifts
+    // known at compile time, but for the smaller of an output's two, which moves
+    // down to the other's unit.  An output stays below 2^room, and what the
+    // first stage of the forward transform adds up, four or three packed complex
+    // values (six where N is an odd multiple of two), below 2^61.  out_sh: the
+    // output's unit and what its two products are moved down by.
+    const int room = N % 4 == 2 ? 57 : 58, drop = 121 - room - kXProd;
+    auto factors = [](int f, int& p, int& q, int& r, int& t) {
+        const int a = MODE == ZFWD ? 0 : (f < 3 ? 3 : 6), b = MODE == ZFWD ? 3 : (f < 3 ? 6 : 0), c = f % 3;
+        p = a + (c + 1) % 3;
+        q = b + (c + 2) % 3;
+        r = a + (c + 2) % 3;
+        t = b + (c + 1) % 3;
     };
-    const int s01 = shift(0, 1), s12 = MODE == ZADJ ? shift(1, 2) : 0, s02 = MODE == ZADJ ? shift(0, 2) : 0;
+    if (threadIdx.x < NOUT) {
+        int p, q, r, t;
+        factors(threadIdx.x, p, q, r, t);
+        const int none = -100000;  // of a product that is 0 everywhere
+        auto top = [&](int f) { return unit(f) + max_sh[f]; };
+        const int t1 = max_sh[p] && max_sh[q] ? top(p) + top(q) : none;
+        const int t2 = max_sh[r] && max_sh[t] ? top(r) + top(t) : none, tm = max(t1, t2);
+        out_sh[threadIdx.x][0] = tm == none ? 0 : tm + 1 - room;
+        out_sh[threadIdx.x][1] = min(tm - t1, 63);
+        out_sh[threadIdx.x][2] = min(tm - t2, 63);
+    }
+    __syncthreads();
+    int up[NIN];
+#pragma unroll
+    for (int f = 0; f < NIN; ++f) up[f] = max(60 - max_sh[f], 0);
+    long long omx[NOUT] = {};
     for (int n = threadIdx.x; n < N; n += blockDim.x) {
-        long long row[2 * NPI];
+        xdig v[2 * NPI];  // the fields' digits
 #pragma unroll
         for (int p = 0; p < NPI; ++p) {
             const fx2 c = ph[at(n, p)];
-            row[2 * p] = c.x;
-            row[2 * p + 1] = c.y;
+            v[2 * p] = x_split(c.x << up[2 * p]);
+            if (2 * p + 1 < NIN) v[2 * p + 1] = x_split(c.y << up[2 * p + 1]);
         }
-        xdig v[NIN], n_[NIN];  // digits of the values and of their negatives
+        long long o[2 * NPO] = {};
 #pragma unroll
-        for (int f = 0; f < NIN; ++f) {
-            v[f] = x_split(row[f]);
-            n_[f] = x_split(-row[f]);
-        }
-        fx2 o[3];
-        if (MODE == ZFWD) {  // u x w
-            o[0] = {cross(v[1], v[5], n_[2], v[4], s01), cross(v[2], v[3], n_[0], v[5], s01)};
-            o[1] = {cross(v[0], v[4], n_[1], v[3], s01), 0};
-        } else {  // w x g, g x u
-            constexpr int g0 = NIN - 3;
-            o[0] = {cross(v[4], v[g0 + 2], n_[5], v[g0 + 1], s12), cross(v[5], v[g0], n_[3], v[g0 + 2], s12)};
-            o[1] = {cross(v[3], v[g0 + 1], n_[4], v[g0], s12), cross(v[g0 + 1], v[2], n_[1], v[g0 + 2], s02)};
-            o[2] = {cross(v[g0 + 2], v[0], n_[2], v[g0], s02), cross(v[g0], v[1], n_[0], v[g0 + 1], s02)};
+        for (int f = 0; f < NOUT; ++f) {
+            int p = 0, q = 0, r = 0, t = 0;
+            factors(f, p, q, r, t);
+            const long long d = (fx_prod(v[p], v[q]) >> out_sh[f][1]) - (fx_prod(v[r], v[t]) >> out_sh[f][2]);
+            o[f] = (d + (1ll << drop >> 1)) >> drop;
+            omx[f] |= o[f] ^ (o[f] >> 63);
         }
 #pragma unroll
-        for (int p = 0; p < NPO; ++p) pr[at(n, p)] = o[p];
+        for (int p = 0; p < NPO; ++p) pr[at(n, p)] = {o[2 * p], o[2 * p + 1]};
+    }
+    {
+        int m[NOUT];
+#pragma unroll
+        for (int f = 0; f < NOUT; ++f) m[f] = __reduce_max_sync(0xffffffffu, x_top(omx[f]));
+        if ((threadIdx.x & 31) == 0)
+#pragma unroll
+            for (int f = 0; f < NOUT; ++f) atomicMax(&omax_sh[f], m[f]);
     }
     __syncthreads();
+    // the bits that the bound left unused (factors of two in each factor, and
+    // maxima that do not meet at one z), usually two to four
+    const xlift lift = {omax_sh, room};
     int halvings = 0;
-    fx2* sp = fx_cols<NPO, NPI, -1, true>(pr, ph, N, tw, &halvings);
+    fx2* sp = fx_cols<NPO, NPI, -1, true>(pr, ph, N, tw, &halvings, &lift);
     const int nan = bad ? 0x7FF80000 : 0;
-    int Eo[2];  // units of the products of the first three outputs and of the others, times 1/2 of the separation
-    Eo[0] = (MODE == ZFWD ? E[0] + E[1] + s01 : E[1] + E[NG - 1] + s12) + 60 - 1 + halvings;
-    Eo[1] = E[0] + E[NG - 1] + s02 + 60 - 1 + halvings;
-    const bool far = Eo[0] < -1000 || Eo[0] > 900 || Eo[1] < -1000 || Eo[1] > 900;
+    const int Eh = halvings - 1;  // the separation's 1/2
+    bool far = false;
+#pragma unroll
+    for (int f = 0; f < NOUT; ++f) {
+        const int e = out_sh[f][0] - lift(f / 2, f % 2) + Eh;
+        far = far || e < -1000 || e > 900;
+    }
     auto put = [&](int f, int k, long long x, long long y) {
-        const int e = Eo[f / 3];
+        const int e = out_sh[f][0] - lift(f / 2, f % 2) + Eh;
         const double s = k == 0 ? sc.o0[f] : sc.ok[f];
         double2 z;
         if (far) z = make_double2(x_store_any(x, e, nan) * s, x_store_any(y, e, nan) * s);
