@@ -1086,29 +1086,50 @@ __device__ __forceinline__ void solve_fixed(XSide& a, const int2* TX, int sh0, i
     const int nan = max(mxb, ou.y) >= 0x7FF00000 ? 0x7FF80000 : 0;
     long long nv[kXR];
     {
-        xdig o[kXR];
+        xdig w[8];  // own four rows, then the other side's
         const int E = max(q.E, ou.x), da = min(E - q.E, 63), db = min(E - ou.x, 63);
 #pragma unroll
         for (int r = 0; r < kXR; ++r) {
             const int2 t = ex[side ^ 1][r][lane];
-            o[r].l = t.x;
-            o[r].h = t.y;
-            o[r] = x_split(x_join(o[r]) >> db);
-            q.w[r] = x_split(x_join(q.w[r]) >> da);
+            xdig o;
+            o.l = t.x;
+            o.h = t.y;
+            w[r] = x_split(x_join(q.w[r]) >> da);
+            w[4 + r] = x_split(x_join(o) >> db);
         }
+        // S^-1 has a third digit and the sums keep 96 bits, to 2^-26 of the unit:
+        // rows of a nearly singular matrix cancel by its condition number
         const int4* G = reinterpret_cast<const int4*>(a.mid) + kk;
+        const int2* G3 = a.mid + 32 * kXK + kk;
+        long long hi[kXR];
+        unsigned lo[kXR];
+        unsigned long long mag = 0;
 #pragma unroll
         for (int r = 0; r < kXR; ++r) {
-            const int4 c0 = G[(r * 4) * kXK], c1 = G[(r * 4 + 1) * kXK], c2 = G[(r * 4 + 2) * kXK], c3 = G[(r * 4 + 3) * kXK];
-            nv[r] = x_dot4(make_int2(c0.x, c0.y), q.w[0], make_int2(c0.z, c0.w), q.w[1], make_int2(c1.x, c1.y), q.w[2],
-                           make_int2(c1.z, c1.w), q.w[3], half) +
-                    x_dot4(make_int2(c2.x, c2.y), o[0], make_int2(c2.z, c2.w), o[1], make_int2(c3.x, c3.y), o[2],
-                           make_int2(c3.z, c3.w), o[3], half);
+            long long H = 0, M = 0, L = 0;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const int4 g = G[(r * 4 + c) * kXK];
+                const int2 t = G3[(r * 4 + c) * kXK];
+                const xdig u = w[2 * c], v = w[2 * c + 1];
+                H = x_mad(g.w, v.h, x_mad(g.y, u.h, H));
+                M = x_mad(g.w, v.l, x_mad(g.z, v.h, x_mad(g.y, u.l, x_mad(g.x, u.h, M))));
+                L = x_mad(t.y, v.h, x_mad(t.x, u.h, L));
+                M += (long long)(int)(x_mul(g.x, u.l) >> 32) + (long long)(int)(x_mul(g.z, v.l) >> 32);
+            }
+            M += L >> 32;
+            hi[r] = H + (M >> 32);
+            lo[r] = (unsigned)M;
+            mag |= (unsigned long long)(hi[r] ^ (hi[r] >> 63));
         }
+        // to 57 bits at most, in units of 2^(32 + d) of the products'
+        const int d = max(64 - __clzll(mag) - 25, 0);
         q.clear();
-        q.E = E + a.mid[32 * kXK + kk].x;
+        q.E = E + a.mid[48 * kXK + kk].x + 32 - kXF + d;
 #pragma unroll
         for (int r = 0; r < kXR; ++r) {
+            const unsigned long long l = (unsigned long long)lo[r] + (1ull << d >> 1);
+            nv[r] = ((hi[r] + (long long)(l >> 32)) << (32 - d)) + (long long)((l & 0xFFFFFFFFull) >> d);
             q.w[r] = x_split(nv[r]);
             q.gw |= x_mag(q.w[r]);
         }
@@ -1212,7 +1233,7 @@ __global__ void __launch_bounds__(64, 6) k_band_solve_x(Geo g, XShape f, const d
                                                         double* __restrict__ pw, const double2* __restrict__ usub) {
     grid_dep_sync();
     __shared__ __align__(16) int2 stage_sh[2][2][kXR * 5 * kXK];
-    __shared__ __align__(16) int2 mid_sh[2][33 * kXK];
+    __shared__ __align__(16) int2 mid_sh[2][kFxMid * kXK];
     __shared__ int2 ex_sh[2][kXR][32], exu_sh[2][32];
     const int nr = g.nr, nht = (g.nk + kXK - 1) / kXK;
     int bi = blockIdx.x;
@@ -1241,7 +1262,7 @@ __global__ void __launch_bounds__(64, 6) k_band_solve_x(Geo g, XShape f, const d
                          (side ? (nr - 1 + a.pad) * rs : 0);
     a.xp = reinterpret_cast<double*>(X + off) + o0;
     a.ad = add ? reinterpret_cast<const double*>(add + off) + o0 : nullptr;
-    for (int i = lane; i < 33 * kXK / 2; i += 32) cp_async16(mid_sh[side] + 2 * i, T + f.mid[side] + 2 * i);
+    for (int i = lane; i < kFxMid * kXK / 2; i += 32) cp_async16(mid_sh[side] + 2 * i, T + f.mid[side] + 2 * i);
     a.stage(0);
     a.load(0);
 

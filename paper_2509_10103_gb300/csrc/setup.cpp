@@ -310,6 +310,12 @@ static double fx_bits(long long c) {
     std::memcpy(&d, &b, sizeof d);
     return d;
 }
+static double fx_pair(int lo, int hi) {
+    const unsigned long long b = ((unsigned long long)(unsigned)hi << 32) | (unsigned)lo;
+    double d;
+    std::memcpy(&d, &b, sizeof d);
+    return d;
+}
 // -a b in fixed point (the product's rounding error included)
 static long long fx_neg(double a, double b) {
     constexpr double s = (double)(1ll << kFxBits);
@@ -317,53 +323,76 @@ static long long fx_neg(double a, double b) {
     return -(std::llround(p * s) + std::llround(e * s));
 }
 
+// Unevaluated sums of two doubles (Dekker 1971, Knuth's two-sum; about 106 bits).
+struct dd {
+    double h = 0.0, l = 0.0;
+};
+static inline dd dd_norm(double h, double l) {  // |l| <= |h|
+    const double s = h + l;
+    return {s, l - (s - h)};
+}
+static inline dd dd_add(dd a, dd b) {
+    const double s = a.h + b.h, v = s - a.h;
+    return dd_norm(s, (a.h - (s - v)) + (b.h - v) + (a.l + b.l));
+}
+static inline dd dd_mul(dd a, dd b) {
+    const double p = a.h * b.h;
+    return dd_norm(p, std::fma(a.h, b.h, -p) + (a.h * b.l + a.l * b.h));
+}
+static inline dd dd_neg(dd a) { return {-a.h, -a.l}; }
+static inline dd dd_inv(dd a) {  // 1 / a, one Newton step
+    const double q = 1.0 / a.h, r = std::fma(-q, a.h, 1.0) - q * a.l;
+    return dd_norm(q, q * r);
+}
+
+// v 2^e as a number with 32 fractional bits: its integer part as two signed digits,
+// the fraction as a third one.
+static double fx_bits(dd v, int e, int& third) {
+    const double h = std::ldexp(v.h, e);
+    long long c = std::llround(h);
+    long long f = std::llround(std::ldexp((h - (double)c) + std::ldexp(v.l, e), 32));  // |h| < 2^53 or h whole
+    c += (f + (1ll << 31)) >> 32;
+    f -= ((f + (1ll << 31)) >> 32) << 32;
+    third = (int)f;
+    const int lo = (int)(unsigned)(c & 0xFFFFFFFFll);
+    return fx_pair(lo, (int)((c - lo) >> 32));
+}
+
 // The two-sided factorisation of one matrix (layout notes in setup.hpp), by
 // positions: l[s][p][e] = N(p, p-4+e) for the outer columns, u[s][p][e] =
 // U(p, p+1+e), d[s][p] = 1/D, all of side s, and the inverse of the middle block.
 struct Twist {
     std::vector<double> l[2], u[2], d[2];
-    double mid[8][8];  // S^-1 by rows h-4..h+3
+    dd mid[8][8];  // S^-1 by rows h-4..h+3
 };
-// G = S^-1: Gauss-Jordan with partial pivoting, then one Newton step
-// G += G (I - S G) with the residual's products and sums compensated.
-static bool invert8(const double (&S)[8][8], double (&G)[8][8]) {
-    double a[8][16];
+// G = S^-1 by Gauss-Jordan elimination with partial pivoting, in place.  The
+// solver multiplies by G instead of solving with S, which is as stable only if
+// G is accurate far beyond the result: nearly singular matrices (the pressure
+// of m = 0 and small k_z in a long pipe, condition number about Lz^2) cancel in
+// G r as many bits as their condition number has.
+static bool invert8(const double (&S)[8][8], dd (&G)[8][8]) {
+    int perm[8];
     for (int i = 0; i < 8; ++i)
-        for (int j = 0; j < 8; ++j) {
-            a[i][j] = S[i][j];
-            a[i][8 + j] = i == j;
-        }
+        for (int j = 0; j < 8; ++j) G[i][j] = {S[i][j], 0.0};
     for (int c = 0; c < 8; ++c) {
         int p = c;
         for (int i = c + 1; i < 8; ++i)
-            if (std::fabs(a[i][c]) > std::fabs(a[p][c])) p = i;
-        if (a[p][c] == 0.0 || !std::isfinite(a[p][c])) return false;
-        if (p != c) std::swap(a[p], a[c]);
-        const double inv = 1.0 / a[c][c];
-        for (int j = c; j < 16; ++j) a[c][j] *= inv;
+            if (std::fabs(G[i][c].h) > std::fabs(G[p][c].h)) p = i;
+        if (G[p][c].h == 0.0 || !std::isfinite(G[p][c].h)) return false;
+        perm[c] = p;
+        for (int j = 0; j < 8 && p != c; ++j) std::swap(G[p][j], G[c][j]);
+        const dd inv = dd_inv(G[c][c]);
+        G[c][c] = {1.0, 0.0};
+        for (int j = 0; j < 8; ++j) G[c][j] = dd_mul(G[c][j], inv);
         for (int i = 0; i < 8; ++i) {
-            const double m = a[i][c];
-            if (i == c || m == 0.0) continue;
-            for (int j = c; j < 16; ++j) a[i][j] = std::fma(-m, a[c][j], a[i][j]);
+            if (i == c) continue;
+            const dd m = dd_neg(G[i][c]);
+            G[i][c] = dd{};
+            for (int j = 0; j < 8; ++j) G[i][j] = dd_add(G[i][j], dd_mul(m, G[c][j]));
         }
     }
-    double R[8][8];
-    for (int i = 0; i < 8; ++i)
-        for (int j = 0; j < 8; ++j) {
-            double s = i == j, e = 0.0;
-            for (int k = 0; k < 8; ++k) {
-                const double p = -S[i][k] * a[k][8 + j], pe = std::fma(-S[i][k], a[k][8 + j], -p), t = s + p, z = t - s;
-                e += ((s - (t - z)) + (p - z)) + pe;
-                s = t;
-            }
-            R[i][j] = s + e;
-        }
-    for (int i = 0; i < 8; ++i)
-        for (int j = 0; j < 8; ++j) {
-            double d = 0.0;
-            for (int k = 0; k < 8; ++k) d = std::fma(a[i][8 + k], R[k][j], d);
-            G[i][j] = a[i][8 + j] + d;
-        }
+    for (int c = 7; c >= 0; --c)  // the row exchanges, undone as column exchanges
+        for (int i = 0; i < 8 && perm[c] != c; ++i) std::swap(G[i][c], G[i][perm[c]]);
     return true;
 }
 static bool twist_factor(const Band& A, const FxShape& f, Twist& t) {
@@ -412,14 +441,22 @@ static bool twist_factor(const Band& A, const FxShape& f, Twist& t) {
 // positions of a side's half of the middle as rows of the block: own, then the other side's
 static int mid_row(int s, int i) { return i < 4 ? (s ? 7 - i : i) : (s ? i - 4 : 11 - i); }
 
-// Residual of the two-sided solve of one random system, relative as in
-// band_backward_error.
+// Backward error of the two-sided solve of A x = b, by rows (Oettli and Prager
+// 1964): the residual over |A||x| + |b|.  b = A x for a random x of order one: the
+// solution of a random b would lie along the null vector of a nearly singular
+// matrix, beside which whatever the middle block loses disappears.
 static double twist_backward_error(const Band& A, const FxShape& f, const Twist& t, unsigned seed) {
     const int n = A.n;
-    std::mt19937_64 g(seed);
-    std::uniform_real_distribution<double> U(-1, 1);
-    std::vector<double> b(n), x(n);
-    for (double& v : b) v = U(g);
+    std::vector<double> b(n, 0.0), x(n);
+    unsigned long long g = seed;
+    for (double& v : x) {  // splitmix64
+        unsigned long long z = g += 0x9E3779B97F4A7C15ull;
+        z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+        z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+        v = 0.5 + std::ldexp((double)((z ^ (z >> 31)) >> 11), -53);
+    }
+    for (int j = 0; j < n; ++j)
+        for (int c = std::max(0, j - kLo); c <= std::min(n - 1, j + kUp); ++c) b[j] += A.get(j, c) * x[c];
     double mid[8];
     std::vector<double> y[2];
     for (int s = 0; s < 2; ++s) {
@@ -437,9 +474,9 @@ static double twist_backward_error(const Band& A, const FxShape& f, const Twist&
         const int np = 4 * f.chunks[s], pad = s ? f.pad : 0;
         std::vector<double> xs(np + 8, 0.0);
         for (int i = 0; i < 4; ++i) {
-            double v = 0;
-            for (int c = 0; c < 8; ++c) v += t.mid[mid_row(s, i)][c] * mid[c];
-            xs[np - 4 + i] = v;
+            dd v;
+            for (int c = 0; c < 8; ++c) v = dd_add(v, dd_mul(t.mid[mid_row(s, i)][c], {mid[c], 0.0}));
+            xs[np - 4 + i] = v.h;
         }
         for (int p = np - 5; p >= pad; --p) {
             double v = y[s][p] * t.d[s][p];
@@ -448,19 +485,17 @@ static double twist_backward_error(const Band& A, const FxShape& f, const Twist&
         }
         for (int p = pad; p < np; ++p) x[s ? n - 1 - (p - pad) : p] = xs[p];
     }
-    double rmax = 0, amax = 0, xmax = 0;
+    double worst = 0;
     for (int j = 0; j < n; ++j) {
-        double r = -b[j], arow = 0;
+        double r = -b[j], arow = std::fabs(b[j]) + 1e-300;
         for (int c = std::max(0, j - kLo); c <= std::min(n - 1, j + kUp); ++c) {
             r += A.get(j, c) * x[c];
-            arow += std::fabs(A.get(j, c));
+            arow += std::fabs(A.get(j, c) * x[c]);
         }
-        rmax = std::max(rmax, std::fabs(r));
-        amax = std::max(amax, arow);
-        xmax = std::max(xmax, std::fabs(x[j]));
+        worst = std::max(worst, std::fabs(r) / arow);
+        if (!std::isfinite(r)) return 1.0;
     }
-    const double e = rmax / (amax * xmax + 1e-300);
-    return std::isfinite(e) ? e : 1.0;
+    return worst;
 }
 
 // Largest row sum of the multipliers of one factorisation (column 0 apart,
@@ -541,13 +576,18 @@ static bool fx_write(FixedTable& tab, int mat, int k, int nht, const FxShape& f,
                 tab.direct[o] = tab.transposed[o] = fx_bits(((scaled - byte + 128) >> 8) * 256 + byte);
             }
         }
-        // S^-1 scaled by a power of two to row sums of at most 1
+        // S^-1 scaled by a power of two to row sums of at most 1, with 32 further
+        // fractional bits in a third digit
         for (int tr = 0; tr < 2; ++tr) {
             auto& dst = tr ? tab.transposed : tab.direct;
+            auto entry = [&](int i, int c) {  // row i of this side, column c: own rows, then the other side's
+                const int a = mid_row(s, i), b = mid_row(s, c);
+                return tr ? t.mid[b][a] : t.mid[a][b];
+            };
             double sum = 0;
             for (int i = 0; i < 4; ++i) {
                 double r = 0;
-                for (int c = 0; c < 8; ++c) r += std::fabs(tr ? t.mid[c][mid_row(s, i)] : t.mid[mid_row(s, i)][c]);
+                for (int c = 0; c < 8; ++c) r += std::fabs(entry(i, c).h);
                 if (!(r <= sum)) sum = r;
             }
             int q = 0;
@@ -556,13 +596,14 @@ static bool fx_write(FixedTable& tab, int mat, int k, int nht, const FxShape& f,
             if (q < -900 || q > 900) return false;
             const size_t o = base + f.mid[s];
             for (int i = 0; i < 4; ++i)
-                for (int c = 0; c < 8; ++c) {
-                    const int a = mid_row(s, i), b = mid_row(s, c);
-                    const double v = tr ? t.mid[b][a] : t.mid[a][b];
-                    dst[o + ((size_t)(i * 4 + c / 2) * kTileX + kk) * 2 + c % 2] =
-                        fx_bits(std::llround(std::ldexp(v, kFxBits - q)));
+                for (int c = 0; c < 8; c += 2) {
+                    int third[2];
+                    for (int e = 0; e < 2; ++e)
+                        dst[o + ((size_t)(i * 4 + c / 2) * kTileX + kk) * 2 + e] =
+                            fx_bits(entry(i, c + e), kFxBits - q, third[e]);
+                    dst[o + ((size_t)(32 + i * 4 + c / 2) * kTileX) + kk] = fx_pair(third[0], third[1]);
                 }
-            dst[o + 32 * kTileX + kk] = fx_bits(q);
+            dst[o + 48 * kTileX + kk] = fx_pair(q, 0);
         }
     }
     for (int i = 0; i < 4; ++i)
@@ -664,7 +705,7 @@ static bool factor_tables(const HostOps& h, FixedTable& t, std::vector<double>& 
             err_t[th] = std::max(err_t[th], band_backward_error(A, f, 1234u + ma * 977u + k));
             each(ma, k, f);
             if (!t.ok || unfit[th]) continue;
-            if (!twist_factor(A, shape, w) || !(twist_backward_error(A, shape, w, 99u + ma * 977u + k) < 1e-12)) {
+            if (!twist_factor(A, shape, w) || !(twist_backward_error(A, shape, w, 99u + ma * 977u + k) < kFxBackward)) {
                 unfit[th] = 1;
                 continue;
             }

@@ -59,7 +59,8 @@ constexpr int kNc1Transposed = kUp + 1;  // A^T x = b rows: U^T (8), 1/diag | L^
 //     [4][k], a 62-bit fixed-point number whose low byte is its exponent, shared
 //     by the rows of a chunk but in the first one; the side's half of S^-1 (or
 //     its transpose), [4][4][k][2] (own four, then the other side's four, in
-//     positions) and its exponent, [k];
+//     positions), the third digits of these entries, [4][4][k] (two 32-bit ones of
+//     one k each), and the exponent, [k];
 //   the wider wall rows, [4][4][k]: columns 5..8 of rows 0..3 of U (direct), rows
 //     0..3 of U for columns 5..8 (transposed).
 // The wall row of A (Dirichlet or Neumann) is not scaled like the others, so
@@ -71,8 +72,14 @@ constexpr int kNc1Transposed = kUp + 1;  // A^T x = b rows: U^T (8), 1/diag | L^
 constexpr int kTileX = 16;
 constexpr int kFxBits = 58;
 constexpr double kFxRowSum = 6.0;
+// largest backward error by rows of a factorisation that is taken (20 roundings of
+// 2^-53; unstretched grids of 21 to 256 points stay below 5e-16 at any Re, dt and
+// length; with the inverse of the middle in one double, 7e-15 at length 8 and
+// 1e-10 at 1000)
+constexpr double kFxBackward = 2e-15;
 constexpr int kFxMinRows = 21;    // smaller grids keep the FP64 solver
 constexpr int kFxMaxChunks = 96;  // chunks of a side the solver keeps units for (768 rows in all)
+constexpr int kFxMid = 49;        // words of a side's middle per k
 struct FixedTable {
     bool ok = false;
     int shift = 0;
@@ -95,7 +102,7 @@ inline FxShape fx_shape(int nr) {
         f.in[s] = at;
         f.out[s] = f.in[s] + n * 16 * kTileX;
         f.mid[s] = f.out[s] + outer * 20 * kTileX;
-        at = f.mid[s] + 33 * kTileX;
+        at = f.mid[s] + kFxMid * kTileX;
     }
     f.wall = at;
     f.tile = f.wall + 16 * kTileX;
