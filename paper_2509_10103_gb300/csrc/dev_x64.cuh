@@ -57,10 +57,18 @@ __device__ __forceinline__ double x_store_any(long long v, int E, int nan) {
     if (f >= 2047) return __hiloint2double((h & (int)0x80000000) | 0x7FF00000, 0);
     return __hiloint2double(h + E * (1 << 20), __double2loint(d));
 }
-// v 2^-n to an integer, n of either sign (the caller bounds left shifts)
-__device__ __forceinline__ long long x_move(long long v, int n) {
-    return (v >> min(max(n, 0), 63)) << min(max(-n, 0), 63);
-}
+// v 2^-n to the nearest integer, n of either sign, |v| < 2^62 (the caller bounds
+// left shifts)
+struct xmove {
+    int right, left;
+    long long half;
+    __device__ __forceinline__ explicit xmove(int n) {
+        right = min(max(n, 0), 62);
+        left = min(max(-n, 0), 62);
+        half = (1ll << right) >> 1;
+    }
+    __device__ __forceinline__ long long operator()(long long v) const { return ((v + half) >> right) << left; }
+};
 
 // signed 32-bit digits: v = h 2^32 + l
 struct xdig {

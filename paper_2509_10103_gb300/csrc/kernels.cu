@@ -853,10 +853,12 @@ __global__ void __launch_bounds__(2 * kSK) k_band_solve(Geo g, const double* __r
 // and the window of the last four results share one exponent, chosen so that
 // the largest has its top bit at 53 or above (a rounding is at most 2^-54 of
 // it, where FP64 arithmetic rounds at 2^-53 of every partial sum) and all stay
-// below 2^60; a chunk whose results outgrow that (a warp vote on their
+// below 2^60; a lane whose results outgrow that in a chunk (seen from their
 // magnitudes, which cannot wrap: one row adds at most a factor 1 + kFxRowSum)
-// is redone with a coarser unit.  Between the sweeps a row stays in fixed point
-// (in place of its right-hand side, each lane reading what it wrote).
+// does the chunk again in units of 2^6.  The exponent is the lane's own (64x64x256:
+// 41.5 us over all solves of a step, 41.6 where a warp vote moved all 32 lanes).
+// Between the sweeps a row stays in fixed point (in place of its right-hand side,
+// each lane reading what it wrote).
 //
 // A block is one (component, m) and 16 consecutive k, a warp per side, lane
 // pairs holding the real and imaginary parts; multipliers stream through the
@@ -875,7 +877,9 @@ struct XShape {
 };
 
 // The window of a sweep: the results of the last chunk (slot i: its row i) and,
-// near the wall, the values only the wall rows read, in units of 2^E.
+// near the wall, the values only the wall rows read, in units of 2^E.  A lane's
+// unit follows its own column alone, so that a mode's rounding does not depend on
+// the others of its tile.
 struct XWin {
     xdig w[4], x[4];
     int gw, gx;  // high-digit magnitudes
@@ -890,18 +894,18 @@ struct XWin {
     }
     __device__ __forceinline__ void coarsen(int d) {  // unit times 2^d
         E += d;
-        const int r = min(max(d, 0), 63), l = min(max(-d, 0), 63);
+        const xmove move(d);
         gw = 0;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            w[i] = x_split((x_join(w[i]) >> r) << l);
+            w[i] = x_split(move(x_join(w[i])));
             gw |= x_mag(w[i]);
         }
         if (wall) {
             gx = 0;
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                x[i] = x_split((x_join(x[i]) >> r) << l);
+                x[i] = x_split(move(x_join(x[i])));
                 gx |= x_mag(x[i]);
             }
         }
@@ -909,7 +913,7 @@ struct XWin {
     // makes room for right-hand sides that need units of at least 2^e
     __device__ __forceinline__ void align(int e) {
         const int mx = gw | gx;
-        if (!__any_sync(0xffffffffu, e > E || mx >= (1 << 26) || (mx < (1 << 21) && e < E - 6))) return;
+        if (!(e > E || mx >= (1 << 26) || (mx < (1 << 21) && e < E - 6))) return;
         int low = 0;
 #pragma unroll
         for (int i = 0; i < 4; ++i) low |= w[i].h | w[i].l | x[i].h | x[i].l;
@@ -1055,7 +1059,7 @@ __device__ __forceinline__ void solve_fixed(XSide& a, const int2* TX, int sh0, i
                 nd[r] = x_split(x_load(b[r], u) + sum);
                 mg |= x_mag(nd[r]);
             }
-            if (!__any_sync(0xffffffffu, mg >= (1 << 28))) break;
+            if (mg < (1 << 28)) break;
             q.coarsen(6);
         }
         q.gw = mg;
@@ -1087,15 +1091,16 @@ __device__ __forceinline__ void solve_fixed(XSide& a, const int2* TX, int sh0, i
     long long nv[kXR];
     {
         xdig w[8];  // own four rows, then the other side's
-        const int E = max(q.E, ou.x), da = min(E - q.E, 63), db = min(E - ou.x, 63);
+        const int E = max(q.E, ou.x);
+        const xmove own(E - q.E), other(E - ou.x);
 #pragma unroll
         for (int r = 0; r < kXR; ++r) {
             const int2 t = ex[side ^ 1][r][lane];
             xdig o;
             o.l = t.x;
             o.h = t.y;
-            w[r] = x_split(x_join(q.w[r]) >> da);
-            w[4 + r] = x_split(x_join(o) >> db);
+            w[r] = x_split(own(x_join(q.w[r])));
+            w[4 + r] = x_split(other(x_join(o)));
         }
         // S^-1 has a third digit and the sums keep 96 bits, to 2^-26 of the unit:
         // rows of a nearly singular matrix cancel by its condition number
@@ -1173,36 +1178,39 @@ __device__ __forceinline__ void solve_fixed(XSide& a, const int2* TX, int sh0, i
                 }
                 e = ez = top - 59;
 #pragma unroll
-                for (int r = 0; r < kXR; ++r) z[r] = x_move(z[r], ez - sr[r]);
+                for (int r = 0; r < kXR; ++r) z[r] = xmove(ez - sr[r])(z[r]);
             }
             if (!TRANS && side == 0 && c == 1) {  // rows 3..0 also read x_5..x_8
                 q.x[3] = q.w[0];
-                q.gx = q.gw;
+                q.gx = x_mag(q.x[3]);
                 q.wall = true;
             }
             if (!TRANS && side == 0 && c == 0) {
 #pragma unroll
-                for (int i = 0; i < 3; ++i) q.x[i] = q.w[i + 1];
-                q.gx |= q.gw;
+                for (int i = 0; i < 3; ++i) {
+                    q.x[i] = q.w[i + 1];
+                    q.gx |= x_mag(q.x[i]);
+                }
             }
             q.align(e);
             xdig nd[kXR];
             int mg;
             for (int tries = 0; tries < 4; ++tries) {
                 const int d = q.E - ez, right = min(max(d, 0), 63), left = min(max(-d, 0), 63);
+                const long long h = right ? 2 * half : half;  // half a unit for what the shift of z cuts off, too
                 mg = 0;
 #pragma unroll
                 for (int r = kXR - 1; r >= 0; --r) {
                     auto win = [&](int i) { return r + i >= 4 ? q.w[(r + i) & 3] : nd[(r + i) & 3]; };  // position p + i
                     const int4 c12 = C[(r * 2) * kXK], c34 = C[(r * 2 + 1) * kXK];
                     long long sum = x_dot4(make_int2(c34.z, c34.w), win(4), make_int2(c34.x, c34.y), win(3),
-                                           make_int2(c12.z, c12.w), win(2), make_int2(c12.x, c12.y), win(1), half);
+                                           make_int2(c12.z, c12.w), win(2), make_int2(c12.x, c12.y), win(1), h);
                     if (!TRANS && side == 0 && c == 0) sum += wall(r);
                     nv[r] = ((z[r] >> right) << left) + sum;
                     nd[r] = x_split(nv[r]);
                     mg |= x_mag(nd[r]);
                 }
-                if (!__any_sync(0xffffffffu, mg >= (1 << 28))) break;
+                if (mg < (1 << 28)) break;
                 q.coarsen(6);
             }
             q.gw = mg;
