@@ -574,7 +574,8 @@ __global__ void __launch_bounds__(256, 3)
     __syncthreads();
     fx2* ph = fx_cols<NPI, NPI, +1>(bufA, bufB, N, tw);
     fx2* pr = ph == bufA ? bufB : bufA;
-    // largest physical values of the fields, for the units of the products
+    // largest physical values of the fields, for the units of the products (a field
+    // that is 0 stays 0, whatever rounding errors its column has)
     {
         long long mx[NIN] = {};
         for (int n = threadIdx.x; n < N; n += blockDim.x) {
@@ -587,7 +588,7 @@ __global__ void __launch_bounds__(256, 3)
         }
         int m[NIN];
 #pragma unroll
-        for (int f = 0; f < NIN; ++f) m[f] = __reduce_max_sync(0xffffffffu, x_top(mx[f]));
+        for (int f = 0; f < NIN; ++f) m[f] = __reduce_max_sync(0xffffffffu, top_sh[f] ? x_top(mx[f]) : 0);
         if ((threadIdx.x & 31) == 0)
 #pragma unroll
             for (int f = 0; f < NIN; ++f) atomicMax(&max_sh[f], m[f]);
@@ -615,14 +616,16 @@ __global__ void __launch_bounds__(256, 3)
         auto top = [&](int f) { return unit(f) + max_sh[f]; };
         const int t1 = max_sh[p] && max_sh[q] ? top(p) + top(q) : none;
         const int t2 = max_sh[r] && max_sh[t] ? top(r) + top(t) : none, tm = max(t1, t2);
-        out_sh[threadIdx.x][0] = tm == none ? 0 : tm + 1 - room;
+        // an output that is 0 stays 0: a unit below the subnormals for the rounding
+        // errors of the one that shares its column
+        out_sh[threadIdx.x][0] = tm == none ? -4000 : tm + 1 - room;
         out_sh[threadIdx.x][1] = min(tm - t1, 63);
         out_sh[threadIdx.x][2] = min(tm - t2, 63);
     }
     __syncthreads();
     int up[NIN];
 #pragma unroll
-    for (int f = 0; f < NIN; ++f) up[f] = max(60 - max_sh[f], 0);
+    for (int f = 0; f < NIN; ++f) up[f] = max_sh[f] ? max(60 - max_sh[f], 0) : 0;
     long long omx[NOUT] = {};
     for (int n = threadIdx.x; n < N; n += blockDim.x) {
         xdig v[2 * NPI];  // the fields' digits

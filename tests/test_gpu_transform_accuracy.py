@@ -77,3 +77,36 @@ def test_transpose_per_component_and_row(env, M, K, scale):
     got, want = apply(L.OP_NONLINEAR_T, u, nb), o.nonlinearT(u, 0.0, nb)
     ctx.close()
     assert float((np.abs(got - want).max(axis=(2, 3)) / np.abs(want).max(axis=(2, 3))).max()) < 2.0 ** -47
+
+
+@pytest.mark.parametrize("e", [-440, -40, -10, 0, 300])
+@pytest.mark.parametrize("M,K", [(1, 127), (2, 26), (8, 17)])
+def test_powers_of_two_and_vanishing_components(env, M, K, e):
+    """u = (0, u_theta, 0) of m = 0: the theta component of u x omega vanishes, exactly, and
+    a factor 2^e on u (a row at the wall being 0) is a factor 2^(2e) on the others."""
+    _, L = env
+    ctx, o, x, apply = setup(env, M, K, (0, 1, 0), M + K)
+    u = x[0]
+    u[:, :, :M] = 0
+    u[:, :, M + 1:] = 0
+    u[:, 0] = 0
+    term = lambda v: 0.5 * apply(L.OP_NONLINEAR, v) + 0.5 * apply(L.OP_NONLINEAR, -v)  # noqa: E731
+    a, b = term(u), term(np.ldexp(u.real, e) + 1j * np.ldexp(u.imag, e))
+    ctx.close()
+    assert np.abs(a[0]).max() > 0.1 and not a[1].any() and not b[1].any()
+    for part in (np.real, np.imag):
+        assert np.array_equal(np.ldexp(part(a), 2 * e), part(b))
+
+
+@pytest.mark.parametrize("e", [-400, -30, 30, 300])
+def test_transpose_in_powers_of_two(env, e):
+    """A factor 2^e on the cotangent, bit for bit, with a row of u that vanishes (g x u is 0
+    there) and a component of the cotangent that does."""
+    _, L = env
+    ctx, o, (u, nb), apply = setup(env, 3, 8, (1, 1, 1), 3)
+    u[:, 0] = 0
+    nb[0, 4] = 0
+    a, b = apply(L.OP_NONLINEAR_T, u, nb), apply(L.OP_NONLINEAR_T, u, np.ldexp(nb.real, e) + 1j * np.ldexp(nb.imag, e))
+    ctx.close()
+    for part in (np.real, np.imag):
+        assert np.array_equal(np.ldexp(part(a), e), part(b))
