@@ -1412,6 +1412,7 @@ pnop::HostOps batch_prepare(const pnop_ctx* c, const pnop_params* p) {
     hs.D1 = c->h.D1;
     hs.D2 = c->h.D2;
     hs.phi = c->h.phi;
+    hs.dphi = c->h.dphi;
     hs.ph = {p->Re, p->Wo, p->A, p->dt, p->tau0};
     std::string err;
     if (!pnop::build_operators(hs, err, true)) throw Status(PNOP_ERR_UNSUPPORTED, err);

@@ -11,7 +11,6 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
-#include <random>
 #include <thread>
 #include <vector>
 
@@ -254,12 +253,23 @@ static void band_solve(int n, const std::vector<double>& f, std::vector<double>&
     }
 }
 
+// Uniform numbers in [0, 1) (splitmix64; a generator with a large state costs more to
+// seed than a banded solve)
+struct Uniform {
+    unsigned long long g;
+    double operator()() {
+        unsigned long long z = g += 0x9E3779B97F4A7C15ull;
+        z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+        z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+        return (double)((z ^ (z >> 31)) >> 11) * 0x1p-53;
+    }
+};
+
 static double band_backward_error(const Band& A, const std::vector<double>& f, unsigned seed) {
     const int n = A.n;
-    std::mt19937_64 g(seed);
-    std::uniform_real_distribution<double> U(-1, 1);
+    Uniform U{seed};
     std::vector<double> b(n), x;
-    for (int j = 0; j < n; ++j) b[j] = U(g);
+    for (int j = 0; j < n; ++j) b[j] = 2.0 * U() - 1.0;
     x = b;
     band_solve(n, f, x);
     double rmax = 0, amax = 0, xmax = 0;
@@ -300,29 +310,6 @@ static std::vector<double> transpose_factors(int nr, const std::vector<double>& 
     return t;
 }
 
-// value in fixed point, as the two signed digits the device reads (low, high)
-static double fx_bits(long long c) {
-    if ((unsigned)(c & 0xFFFFFFFFll) == 0x80000000u) ++c;  // keeps the low digit above -2^31 (x_dot4's sums)
-    const int lo = (int)(unsigned)(c & 0xFFFFFFFFll);
-    const unsigned hi = (unsigned)(int)((c - lo) >> 32);
-    const unsigned long long b = ((unsigned long long)hi << 32) | (unsigned)lo;
-    double d;
-    std::memcpy(&d, &b, sizeof d);
-    return d;
-}
-static double fx_pair(int lo, int hi) {
-    const unsigned long long b = ((unsigned long long)(unsigned)hi << 32) | (unsigned)lo;
-    double d;
-    std::memcpy(&d, &b, sizeof d);
-    return d;
-}
-// -a b in fixed point (the product's rounding error included)
-static long long fx_neg(double a, double b) {
-    constexpr double s = (double)(1ll << kFxBits);
-    const double p = a * b, e = std::fma(a, b, -p);
-    return -(std::llround(p * s) + std::llround(e * s));
-}
-
 // Unevaluated sums of two doubles (Dekker 1971, Knuth's two-sum; about 106 bits).
 struct dd {
     double h = 0.0, l = 0.0;
@@ -345,12 +332,69 @@ static inline dd dd_inv(dd a) {  // 1 / a, one Newton step
     return dd_norm(q, q * r);
 }
 
-// v 2^e as a number with 32 fractional bits: its integer part as two signed digits,
-// the fraction as a third one.
-static double fx_bits(dd v, int e, int& third) {
-    const double h = std::ldexp(v.h, e);
-    long long c = std::llround(h);
-    long long f = std::llround(std::ldexp((h - (double)c) + std::ldexp(v.l, e), 32));  // |h| < 2^53 or h whole
+// s + sum a_i x_i with the roundings of the products and sums carried along
+static inline double dd_dot(double s, int n, const double* a, double sign, const dd* x) {
+    double c = 0.0;
+    for (int i = 0; i < n; ++i) {
+        const double ai = sign * a[i], p = ai * x[i].h, t = s + p, z = t - s;
+        c += ((s - (t - z)) + (p - z)) + std::fma(ai, x[i].h, -p) + ai * x[i].l;
+        s = t;
+    }
+    return s + c;
+}
+// x <- A^-1 e_0 by the factors f of A and refinement with exact residuals, until a
+// correction stays below the last bits of x.
+static void unit_response(const Band& A, const std::vector<double>& f, std::vector<dd>& x) {
+    const int n = A.n;
+    std::vector<double> r(n, 0.0);
+    r[0] = 1.0;
+    band_solve(n, f, r);
+    x.assign(n, dd{});
+    for (int rounds = 0;; ++rounds) {
+        double step = 0, size = 0;
+        for (int j = 0; j < n; ++j) {
+            x[j] = dd_add(x[j], {r[j], 0.0});
+            step = std::max(step, std::fabs(r[j]));
+            size = std::max(size, std::fabs(x[j].h));
+        }
+        if (rounds == 3 || (rounds && !(step > std::ldexp(size, -50)))) return;
+        for (int j = 0; j < n; ++j) {
+            const int lo = std::max(0, j - kLo), hi = std::min(n - 1, j + kUp);
+            r[j] = dd_dot(j == 0 ? 1.0 : 0.0, hi - lo + 1, &A.a[(size_t)j * kBand + (lo - j + kLo)], -1.0, &x[lo]);
+        }
+        band_solve(n, f, r);
+    }
+}
+
+// value in fixed point, as the two signed digits the device reads (low, high)
+static double fx_bits(long long c) {
+    if ((unsigned)(c & 0xFFFFFFFFll) == 0x80000000u) ++c;  // keeps the low digit above -2^31 (x_dot4's sums)
+    const int lo = (int)(unsigned)(c & 0xFFFFFFFFll);
+    const unsigned hi = (unsigned)(int)((c - lo) >> 32);
+    const unsigned long long b = ((unsigned long long)hi << 32) | (unsigned)lo;
+    double d;
+    std::memcpy(&d, &b, sizeof d);
+    return d;
+}
+static double fx_pair(int lo, int hi) {
+    const unsigned long long b = ((unsigned long long)(unsigned)hi << 32) | (unsigned)lo;
+    double d;
+    std::memcpy(&d, &b, sizeof d);
+    return d;
+}
+// v scale to the nearest integer, scale a power of two (halves away from zero)
+static inline long long fx_near(double v) { return (long long)(v + std::copysign(0.5, v)); }
+static inline long long fx_round(dd v, double scale) {
+    const double h = v.h * scale;
+    const long long c = std::fabs(h) < 4503599627370496.0 ? fx_near(h) : (long long)h;  // whole from 2^52 on
+    return c + fx_near((h - (double)c) + v.l * scale);
+}
+
+// v scale as a number with 32 fractional bits: its integer part as two signed digits,
+// the fraction as a third one
+static double fx_bits(dd v, double scale, int& third) {
+    long long c = (long long)(v.h * scale);
+    long long f = fx_round({v.h * scale - (double)c, v.l * scale}, 4294967296.0);
     c += (f + (1ll << 31)) >> 32;
     f -= ((f + (1ll << 31)) >> 32) << 32;
     third = (int)f;
@@ -361,19 +405,21 @@ static double fx_bits(dd v, int e, int& third) {
 // The two-sided factorisation of one matrix (layout notes in setup.hpp), by
 // positions: l[s][p][e] = N(p, p-4+e) for the outer columns, u[s][p][e] =
 // U(p, p+1+e), d[s][p] = 1/D, all of side s, and the inverse of the middle block.
+// Computed in sums of two doubles and rounded once, into the tables: in FP64 the
+// elimination and the scaling by 1/D leave several roundings of 2^-53 in every
+// factor, which the solver, rounding at 2^-54 and below, would repeat in every
+// solve.
 struct Twist {
-    std::vector<double> l[2], u[2], d[2];
+    std::vector<dd> l[2], u[2], d[2];
     dd mid[8][8];  // S^-1 by rows h-4..h+3
 };
-// G = S^-1 by Gauss-Jordan elimination with partial pivoting, in place.  The
+// G <- G^-1 by Gauss-Jordan elimination with partial pivoting.  The
 // solver multiplies by G instead of solving with S, which is as stable only if
 // G is accurate far beyond the result: nearly singular matrices (the pressure
 // of m = 0 and small k_z in a long pipe, condition number about Lz^2) cancel in
 // G r as many bits as their condition number has.
-static bool invert8(const double (&S)[8][8], dd (&G)[8][8]) {
+static bool invert8(dd (&G)[8][8]) {
     int perm[8];
-    for (int i = 0; i < 8; ++i)
-        for (int j = 0; j < 8; ++j) G[i][j] = {S[i][j], 0.0};
     for (int c = 0; c < 8; ++c) {
         int p = c;
         for (int i = c + 1; i < 8; ++i)
@@ -397,46 +443,46 @@ static bool invert8(const double (&S)[8][8], dd (&G)[8][8]) {
 }
 static bool twist_factor(const Band& A, const FxShape& f, Twist& t) {
     const int n = A.n, h = f.h, B = 8, W = 2 * B + 1;
-    thread_local std::vector<double> w;
-    w.assign((size_t)n * W, 0.0);
-    auto at = [&](int i, int j) -> double& { return w[(size_t)i * W + (j - i + B)]; };
+    thread_local std::vector<dd> w;
+    w.assign((size_t)n * W, dd{});
+    auto at = [&](int i, int j) -> dd& { return w[(size_t)i * W + (j - i + B)]; };
     for (int i = 0; i < n; ++i)
-        for (int j = std::max(0, i - kLo); j <= std::min(n - 1, i + kUp); ++j) at(i, j) = A.get(i, j);
+        for (int j = std::max(0, i - kLo); j <= std::min(n - 1, i + kUp); ++j) at(i, j).h = A.get(i, j);
     for (int s = 0; s < 2; ++s) {
         const int np = 4 * f.chunks[s], pad = s ? f.pad : 0;
-        t.l[s].assign((size_t)np * 4, 0.0);
-        t.u[s].assign((size_t)np * 8, 0.0);
-        t.d[s].assign(np, 0.0);
+        t.l[s].assign((size_t)np * 4, dd{});
+        t.u[s].assign((size_t)np * 8, dd{});
+        t.d[s].assign(np, dd{});
         auto row = [&](int p) { return s ? n - 1 - (p - pad) : p; };
         for (int p = pad; p < np - 4; ++p) {
             const int i = row(p);
-            const double piv = at(i, i);
-            if (piv == 0.0 || !std::isfinite(piv)) return false;
-            t.d[s][p] = 1.0 / piv;
+            const dd piv = at(i, i);
+            if (piv.h == 0.0 || !std::isfinite(piv.h)) return false;
+            const dd inv = t.d[s][p] = dd_inv(piv);
             for (int e = 0; e < 8; ++e) {
                 const int q = p + 1 + e, j = row(q);
                 if (j < 0 || j >= n) break;
-                const double v = at(i, j);
-                if (v != 0.0 && e >= 4 && (s || p > 3 || q > 8)) return false;
-                t.u[s][(size_t)p * 8 + e] = v * t.d[s][p];
+                const dd v = at(i, j);
+                if (v.h != 0.0 && e >= 4 && (s || p > 3 || q > 8)) return false;
+                t.u[s][(size_t)p * 8 + e] = dd_mul(v, inv);
             }
             for (int q = p + 1; q <= p + 4; ++q) {
                 const int j = row(q);
-                const double m = at(j, i) / piv;
+                const dd m = dd_mul(at(j, i), inv);
                 t.l[s][(size_t)q * 4 + (p - q + 4)] = m;
-                if (m == 0.0) continue;
+                if (m.h == 0.0) continue;
+                const dd neg = dd_neg(m);
                 for (int c = 1; c <= 8; ++c) {
                     const int k = row(p + c);
                     if (k < 0 || k >= n || std::abs(k - j) > B) break;
-                    at(j, k) -= m * at(i, k);
+                    if (at(i, k).h != 0.0) at(j, k) = dd_add(at(j, k), dd_mul(neg, at(i, k)));
                 }
             }
         }
     }
-    double S[8][8];
     for (int i = 0; i < 8; ++i)
-        for (int j = 0; j < 8; ++j) S[i][j] = at(h - 4 + i, h - 4 + j);
-    return invert8(S, t.mid);
+        for (int j = 0; j < 8; ++j) t.mid[i][j] = at(h - 4 + i, h - 4 + j);
+    return invert8(t.mid);
 }
 // positions of a side's half of the middle as rows of the block: own, then the other side's
 static int mid_row(int s, int i) { return i < 4 ? (s ? 7 - i : i) : (s ? i - 4 : 11 - i); }
@@ -448,13 +494,8 @@ static int mid_row(int s, int i) { return i < 4 ? (s ? 7 - i : i) : (s ? i - 4 :
 static double twist_backward_error(const Band& A, const FxShape& f, const Twist& t, unsigned seed) {
     const int n = A.n;
     std::vector<double> b(n, 0.0), x(n);
-    unsigned long long g = seed;
-    for (double& v : x) {  // splitmix64
-        unsigned long long z = g += 0x9E3779B97F4A7C15ull;
-        z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-        z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-        v = 0.5 + std::ldexp((double)((z ^ (z >> 31)) >> 11), -53);
-    }
+    Uniform U{seed};
+    for (double& v : x) v = 0.5 + U();
     for (int j = 0; j < n; ++j)
         for (int c = std::max(0, j - kLo); c <= std::min(n - 1, j + kUp); ++c) b[j] += A.get(j, c) * x[c];
     double mid[8];
@@ -465,7 +506,7 @@ static double twist_backward_error(const Band& A, const FxShape& f, const Twist&
         for (int p = pad; p < np; ++p) {
             double v = b[s ? n - 1 - (p - pad) : p];
             for (int e = 0; e < 4; ++e)
-                if (p - 4 + e >= 0) v -= t.l[s][(size_t)p * 4 + e] * y[s][p - 4 + e];
+                if (p - 4 + e >= 0) v -= t.l[s][(size_t)p * 4 + e].h * y[s][p - 4 + e];
             y[s][p] = v;
         }
         for (int i = 0; i < 4; ++i) mid[mid_row(s, i)] = y[s][np - 4 + i];
@@ -479,8 +520,8 @@ static double twist_backward_error(const Band& A, const FxShape& f, const Twist&
             xs[np - 4 + i] = v.h;
         }
         for (int p = np - 5; p >= pad; --p) {
-            double v = y[s][p] * t.d[s][p];
-            for (int e = 0; e < 8; ++e) v -= t.u[s][(size_t)p * 8 + e] * xs[p + 1 + e];
+            double v = y[s][p] * t.d[s][p].h;
+            for (int e = 0; e < 8; ++e) v -= t.u[s][(size_t)p * 8 + e].h * xs[p + 1 + e];
             xs[p] = v;
         }
         for (int p = pad; p < np; ++p) x[s ? n - 1 - (p - pad) : p] = xs[p];
@@ -506,18 +547,18 @@ static void fx_measure(const FxShape& f, const Twist& t, double& sum, double& co
         for (int p = 0; p < np; ++p) {
             double l = 0, u = 0, lt = 0, ut = 0;  // rows and columns of N and U
             for (int e = 0; e < 4; ++e) {
-                const double a = std::fabs(t.l[s][(size_t)p * 4 + e]);
+                const double a = std::fabs(t.l[s][(size_t)p * 4 + e].h);
                 const bool first = s == 0 && p - 4 + e == 0;
                 if (first) col0 = std::max(col0, a);
                 l += first ? std::min(a, 1.0) : a;
                 if (p + 1 + e < np) {
-                    const double b = std::fabs(t.l[s][(size_t)(p + 1 + e) * 4 + 3 - e]);
+                    const double b = std::fabs(t.l[s][(size_t)(p + 1 + e) * 4 + 3 - e].h);
                     lt += s == 0 && p == 0 ? std::min(b, 1.0) : b;
                 }
             }
             for (int e = 0; e < 8; ++e) {
-                u += std::fabs(t.u[s][(size_t)p * 8 + e]);
-                if (p - 1 - e >= 0) ut += std::fabs(t.u[s][(size_t)(p - 1 - e) * 8 + e]);
+                u += std::fabs(t.u[s][(size_t)p * 8 + e].h);
+                if (p - 1 - e >= 0) ut += std::fabs(t.u[s][(size_t)(p - 1 - e) * 8 + e].h);
             }
             const double worst = std::max(std::max(l, u), std::max(lt, ut));
             if (!(worst <= sum)) sum = worst;  // NaN included
@@ -529,15 +570,16 @@ static void fx_measure(const FxShape& f, const Twist& t, double& sum, double& co
 // outside the range of its format.
 static bool fx_write(FixedTable& tab, int mat, int k, int nht, const FxShape& f, const Twist& t) {
     const size_t base = ((size_t)mat * nht + k / kTileX) * f.tile, kk = k % kTileX;
-    auto mult = [&](double v, double scale) { return fx_bits(fx_neg(v, scale)); };
+    const double one = std::ldexp(1.0, kFxBits), col0 = std::ldexp(1.0, kFxBits - tab.shift);
+    auto mult = [&](dd v, double scale) { return fx_bits(fx_round(dd_neg(v), scale)); };
     auto pair = [&](size_t row, int e) { return ((row * 2 + e / 2) * kTileX + kk) * 2 + e % 2; };
     for (int s = 0; s < 2; ++s) {
         const int np = 4 * f.chunks[s];
         auto L = [&](int p, int q) {  // N(p, q), q < p
             const bool first = s == 0 && q == 0;
-            return q < 0 || p >= np ? 0.0 : mult(t.l[s][(size_t)p * 4 + (q - p + 4)], first ? std::ldexp(1.0, -tab.shift) : 1.0);
+            return q < 0 || p >= np ? 0.0 : mult(t.l[s][(size_t)p * 4 + (q - p + 4)], first ? col0 : one);
         };
-        auto U = [&](int p, int q) { return p < 0 || q >= np ? 0.0 : mult(t.u[s][(size_t)p * 8 + (q - p - 1)], 1.0); };
+        auto U = [&](int p, int q) { return p < 0 || q >= np ? 0.0 : mult(t.u[s][(size_t)p * 8 + (q - p - 1)], one); };
         for (int p = 0; p < np; ++p) {
             const size_t in = base + f.in[s], out = base + f.out[s] + (size_t)(p / 4) * 20 * kTileX;
             for (int e = 0; e < 4; ++e) {
@@ -562,16 +604,17 @@ static bool fx_write(FixedTable& tab, int mat, int k, int nht, const FxShape& f,
             int lo = 1 << 20, hi = -(1 << 20);
             for (int i = p; i < end; ++i) {
                 int q = 0;
-                std::frexp(t.d[s][i], &q);
-                if (t.d[s][i] == 0.0) continue;  // empty position
+                std::frexp(t.d[s][i].h, &q);
+                if (t.d[s][i].h == 0.0) continue;  // empty position
                 lo = std::min(lo, q);
                 hi = std::max(hi, q);
             }
             if (lo > hi) lo = hi = 0;
             const int q = hi - 2;
             if (hi - lo > 6 || q < -127 || q > 127) return false;
+            const double unit = std::ldexp(1.0, 60 - q);
             for (; p < end; ++p) {
-                const long long scaled = std::llround(std::ldexp(t.d[s][p], 60 - q)), byte = q + 128;
+                const long long scaled = fx_round(t.d[s][p], unit), byte = q + 128;
                 const size_t o = base + f.out[s] + (size_t)(p / 4) * 20 * kTileX + (16 + p % 4) * kTileX + kk;
                 tab.direct[o] = tab.transposed[o] = fx_bits(((scaled - byte + 128) >> 8) * 256 + byte);
             }
@@ -595,12 +638,13 @@ static bool fx_write(FixedTable& tab, int mat, int k, int nht, const FxShape& f,
             std::frexp(sum, &q);
             if (q < -900 || q > 900) return false;
             const size_t o = base + f.mid[s];
+            const double unit = std::ldexp(1.0, kFxBits - q);
             for (int i = 0; i < 4; ++i)
                 for (int c = 0; c < 8; c += 2) {
                     int third[2];
                     for (int e = 0; e < 2; ++e)
                         dst[o + ((size_t)(i * 4 + c / 2) * kTileX + kk) * 2 + e] =
-                            fx_bits(entry(i, c + e), kFxBits - q, third[e]);
+                            fx_bits(entry(i, c + e), unit, third[e]);
                     dst[o + ((size_t)(32 + i * 4 + c / 2) * kTileX) + kk] = fx_pair(third[0], third[1]);
                 }
             dst[o + 48 * kTileX + kk] = fx_pair(q, 0);
@@ -609,7 +653,7 @@ static bool fx_write(FixedTable& tab, int mat, int k, int nht, const FxShape& f,
     for (int i = 0; i < 4; ++i)
         for (int e = 0; e < 4; ++e) {  // U(i, 5 + e), the part beyond four columns
             const int c = 5 + e;
-            const double v = c - i > 4 ? mult(t.u[0][(size_t)i * 8 + (c - i - 1)], 1.0) : 0.0;
+            const double v = c - i > 4 ? mult(t.u[0][(size_t)i * 8 + (c - i - 1)], one) : 0.0;
             tab.direct[base + f.wall + (size_t)(i * 4 + e) * kTileX + kk] = v;
             tab.transposed[base + f.wall + (size_t)(e * 4 + i) * kTileX + kk] = v;
         }
@@ -703,7 +747,7 @@ static bool factor_tables(const HostOps& h, FixedTable& t, std::vector<double>& 
                 return;
             }
             err_t[th] = std::max(err_t[th], band_backward_error(A, f, 1234u + ma * 977u + k));
-            each(ma, k, f);
+            each(ma, k, A, f);
             if (!t.ok || unfit[th]) continue;
             if (!twist_factor(A, shape, w) || !(twist_backward_error(A, shape, w, 99u + ma * 977u + k) < kFxBackward)) {
                 unfit[th] = 1;
@@ -762,13 +806,16 @@ bool build_operators(HostOps& h, std::string& err, bool reuse_pressure) {
     }
     h.ntile = (nk + kTileK - 1) / kTileK;
     double worst = 0;
-    // Pressure factors, and the pressure phi of a unit wall datum for every
-    // (|m|, k): they depend on the grid only, a caller that built them for this
-    // grid before may keep them.
+    // Pressure factors, and the pressure phi of a unit wall datum with its radial
+    // derivative for every (|m|, k): they depend on the grid only, a caller that
+    // built them for this grid before may keep them.  They are as accurate as the
+    // solver's tables (an LU alone leaves 2^-53 times the condition number, about
+    // Lz^2 for m = 0, k = 1, and the wall correction would not match the solves).
     const size_t sys = (size_t)(M + 1) * nk * nr;
     auto at = [&](int ma, int k) { return ((size_t)ma * nk + k) * nr; };
     if (!(reuse_pressure && h.phi.size() == sys)) {
         h.phi.assign(sys, 0.0);
+        h.dphi.assign(sys, 0.0);
         const bool done = factor_tables(
             h, h.fxP, h.facP, h.facPT, M + 1,
             [&](int ma, double kz) {
@@ -777,12 +824,16 @@ bool build_operators(HostOps& h, std::string& err, bool reuse_pressure) {
                 for (int j = 0; j < nr; ++j) I.at(j, j) = 1.0;
                 return I;
             },
-            [&](int ma, int k, const std::vector<double>& f) {
+            [&](int ma, int k, const Band& A, const std::vector<double>& f) {
                 if (ma == 0 && k == 0) return;
-                std::vector<double> x(nr, 0.0);
-                x[0] = 1.0;
-                band_solve(nr, f, x);
-                std::copy(x.begin(), x.end(), h.phi.begin() + at(ma, k));
+                thread_local std::vector<dd> x;
+                unit_response(A, f, x);
+                for (int j = 0; j < nr; ++j) {
+                    const int lo = std::max(0, j - kLo), hi = std::min(nr - 1, j + kUp);
+                    const double* row = &h.D1[((size_t)parity_index(ma) * nr + j) * kBand + (lo - j + kLo)];
+                    h.phi[at(ma, k) + j] = x[j].h;
+                    h.dphi[at(ma, k) + j] = dd_dot(0.0, hi - lo + 1, row, 1.0, &x[lo]);
+                }
             },
             worst);
         if (!done) {
@@ -796,23 +847,14 @@ bool build_operators(HostOps& h, std::string& err, bool reuse_pressure) {
     std::vector<double> hp(sys, 0.0), hm(sys, 0.0), hz(sys, 0.0);
     const bool done = factor_tables(
         h, h.fxH, h.facH, h.facHT, M + 2, [&](int ma, double kz) { return helmholtz_band(h, ma, kz); },
-        [&](int mu, int k, const std::vector<double>& f) {
+        [&](int mu, int k, const Band&, const std::vector<double>& f) {
             const double kz = 2.0 * M_PI * k / d.Lz;
             std::vector<double> x(nr);
             auto solve = [&](int m, int kind, std::vector<double>& to) {  // kind +1, -1: u+-, 0: u_z
                 if (m < 0 || m > M || (m == 0 && k == 0)) return;
-                const double* phi = &h.phi[at(m, k)];
-                const int pp = parity_index(m);
-                for (int j = 0; j < nr; ++j) {
-                    if (kind == 0) {
-                        x[j] = -kz * phi[j];
-                        continue;
-                    }
-                    double dphi = 0;
-                    for (int c = std::max(0, j - kLo); c <= std::min(nr - 1, j + kUp); ++c)
-                        dphi += h.D1[((size_t)pp * nr + j) * kBand + (c - j + kLo)] * phi[c];
-                    x[j] = -dphi + kind * m * h.invr[j] * phi[j];
-                }
+                const double *phi = &h.phi[at(m, k)], *dphi = &h.dphi[at(m, k)];
+                for (int j = 0; j < nr; ++j)
+                    x[j] = kind == 0 ? -kz * phi[j] : -dphi[j] + kind * m * h.invr[j] * phi[j];
                 x[0] = 0.0;
                 band_solve(nr, f, x);
                 std::copy(x.begin(), x.end(), to.begin() + at(m, k));

@@ -125,7 +125,7 @@ struct HostOps {
     int ntile = 0;
     FixedTable fxH, fxP;
     std::vector<double> facH, facHT, facP, facPT;
-    std::vector<double> phi;                    // [M+1][nk][nr] pressure of a unit wall datum
+    std::vector<double> phi, dphi;              // [M+1][nk][nr] pressure of a unit wall datum, its radial derivative
     std::vector<double> infl;                   // [nm][3][nr][nk] influence response, pre-scaled by -1/delta
     std::vector<double> fluxg;                  // [nr] flux response of mode (0,0)
     double flux_inv = 0;                        // 1 / sum_j W_j g_j
@@ -138,7 +138,7 @@ int parity_index(int m);  // 0 when m is even, 1 when odd
 // Builds grid, weights and finite differences (Re-independent part).
 bool build_grid(HostOps& h, std::string& err);
 // Builds base flow, banded LU factors, influence and flux vectors.
-// reuse_pressure: keep h.phi, and leave the pressure tables alone, when it
+// reuse_pressure: keep h.phi and h.dphi, and leave the pressure tables alone, when it
 // already has this grid's size (they depend on the grid only, not on Re or dt).
 bool build_operators(HostOps& h, std::string& err, bool reuse_pressure = false);
 
