@@ -288,9 +288,7 @@ void upload_slot_operators(pnop_ctx* c, int slot, const pnop::HostOps& h) {
         c->geo.sNk = dg.size();
     }
     // banded factors: a slot's table has room for either form
-    const size_t nht = (h.d.nk + pnop::kTileX - 1) / pnop::kTileX, tile = nht * pnop::fx_shape(h.d.nr).tile;
-    const size_t fp64 = (size_t)h.ntile * h.d.nr * pnop::kBand * pnop::kTileK;
-    const size_t strideH = (h.d.M + 2) * std::max(fp64, tile), strideP = (h.d.M + 1) * std::max(fp64, tile);
+    const size_t words = pnop::factor_words(h.d.nr, h.d.nk), strideH = (h.d.M + 2) * words, strideP = (h.d.M + 1) * words;
     put(c->d_facH, h.fxH.ok ? h.fxH.direct : h.facH, ns, slot, strideH);
     put(c->d_facHT, h.fxH.ok ? h.fxH.transposed : h.facHT, ns, slot, strideH);
     c->geo.sFacH = strideH;
@@ -1561,13 +1559,13 @@ int pnop_context_bytes(const pnop_grid* grid, const pnop_params* params, int sna
     if (!grid || !params || !bytes || snaps < 1 || grid->nr < 1 || grid->ntheta < 4 || grid->nz < 4)
         return PNOP_ERR_INVALID_ARG;
     const size_t nr = grid->nr, M = grid->ntheta / 2 - 1, K = grid->nz / 2 - 1;
-    const size_t nm = 2 * M + 1, nk = K + 1, nkp = (nk + pnop::kTileK - 1) / pnop::kTileK * pnop::kTileK, nt = 3 * (M + 1);
+    const size_t nm = 2 * M + 1, nk = K + 1, nt = 3 * (M + 1);
     const size_t S = nr * nm * nk, field = 3 * S * 16;
     const size_t cz = (params->precision & PNOP_MIXED) ? 8 : 16;
     size_t b = (21 + (size_t)snaps) * field + 2 * S * 16;              // work fields, u_N, optimiser, host staging, checkpoints, q, q2
     b += 24 * nr * nt * nk * cz;                                         // transform scratch Y, Y2, Z
     b += 10 * field + S * 16 + 15 * nr * nt * nk * cz;                   // recomputation workspace (shadow) and its scratch states
-    b += 2 * ((M + 2) + (M + 1)) * nr * 13 * nkp * 8;                    // LU factors and transposed rows
+    b += 2 * ((M + 2) + (M + 1)) * pnop::factor_words(grid->nr, (int)nk) * 8;  // banded factors, direct and transposed
     b += (M + 2) * nr * 13 * 8 + 2 * nr * 13 * 8 + nm * nk * 3 * nr * 8; // bands, D1, influence
     *bytes = b + (1 << 20) + (40 + (size_t)snaps) * (2 << 20);        // tables, reductions, allocation rounding
     return PNOP_OK;
@@ -1584,12 +1582,12 @@ int pnop_batch_bytes(const pnop_grid* grid, const pnop_params* params, int capac
         grid->nr < 1 || grid->ntheta < 4 || grid->nz < 4)
         return PNOP_ERR_INVALID_ARG;
     const size_t nr = grid->nr, M = grid->ntheta / 2 - 1, K = grid->nz / 2 - 1, C = capacity;
-    const size_t nm = 2 * M + 1, nk = K + 1, nkp = (nk + pnop::kTileK - 1) / pnop::kTileK * pnop::kTileK, nt = 3 * (M + 1);
+    const size_t nm = 2 * M + 1, nk = K + 1, nt = 3 * (M + 1);
     const size_t S = nr * nm * nk, field = 3 * S * 16, snaps = (size_t)params->snap_budget;
     const size_t cz = (params->precision & PNOP_MIXED) ? 8 : 16;
     size_t b = C * (18 + snaps) * field;                                 // work fields, state, cotangent, result, q, q2, checkpoints
     b += C * 27 * nr * nt * nk * cz;                                     // transform scratch Y, Y2, Z (9 planes each)
-    b += C * 2 * (M + 2) * nr * 13 * nkp * 8 + 2 * (M + 1) * nr * 13 * nkp * 8;  // Helmholtz factors per slot, pressure shared
+    b += (C * 2 * (M + 2) + 2 * (M + 1)) * pnop::factor_words(grid->nr, (int)nk) * 8;  // Helmholtz factors per slot, pressure shared
     b += C * ((M + 2) * nr * 13 * 8 + nm * nk * 3 * nr * 8 + nk * 8 + 5 * nr * 8) + 2 * nr * 13 * 8;  // bands, influence
     *bytes = b + (1 << 20) + C * (40 + snaps) * (2 << 20);              // tables, reductions, allocation rounding
     return PNOP_OK;

@@ -109,6 +109,14 @@ inline FxShape fx_shape(int nr) {
     return f;
 }
 
+// Words of one matrix's table, room for either form (on grids of 21 and 22 points
+// the fixed-point one is the longer).
+inline size_t factor_words(int nr, int nk) {
+    const size_t fp64 = (size_t)((nk + kTileK - 1) / kTileK) * nr * kBand * kTileK;
+    const size_t fixed = (size_t)((nk + kTileX - 1) / kTileX) * fx_shape(nr).tile;
+    return fp64 > fixed ? fp64 : fixed;
+}
+
 // Everything the device needs, laid out for coalesced access across k.
 struct HostOps {
     Dims d;

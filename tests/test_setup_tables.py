@@ -5,6 +5,7 @@ program that checks what it builds against 113-bit arithmetic.
   of, is rounded once (2^-52 of its largest value, however close to singular the
   matrix is);
 - the multipliers of the two-sided factorisation are rounded once, to 2^-58;
+- the space that contexts reserve and report for the tables holds either form;
 - which grids the integer solver takes: every unstretched one of 21 to 768
   radial points at any Reynolds number, time step and length, and no other size;
   stretched ones by their row sums."""
@@ -133,6 +134,15 @@ int main(int argc, char** argv) {
         const HostOps s = build(32, 2, 5, 8.0, 1800.0, 0.005, 0.1);  // wide stencils: sums above kFxRowSum
         return s.fxP.ok || !s.fxH.ok || s.facP.empty() || !s.facH.empty();
     }
+    if (what == "sizes") {
+        for (int nr = 9; nr <= 800; ++nr)
+            for (int nk : {2, 16, 17, 32, 33, 128, 129})
+                if (factor_words(nr, nk) < (nk + kTileX - 1) / kTileX * fx_shape(nr).tile ||
+                    factor_words(nr, nk) < (size_t)((nk + kTileK - 1) / kTileK) * nr * kBand * kTileK)
+                    return 1;
+        const HostOps h = build(21, 2, 31, 8.0, 1800.0, 0.005, 0.0);
+        return !(h.fxP.direct.size() <= 3 * factor_words(21, 32) && h.fxH.transposed.size() <= 4 * factor_words(21, 32));
+    }
     return 4;
 }
 """
@@ -150,7 +160,7 @@ def program(tmp_path_factory):
     return str(exe)
 
 
-@pytest.mark.parametrize("what", ["response", "multipliers", "grids"])
+@pytest.mark.parametrize("what", ["response", "multipliers", "grids", "sizes"])
 def test_tables(program, what):
     p = subprocess.run([program, what], stdout=subprocess.PIPE, text=True, timeout=600)
     assert p.returncode == 0, p.stdout
