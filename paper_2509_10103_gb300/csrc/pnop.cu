@@ -266,7 +266,7 @@ std::vector<int4> twiddle_digits(int N) {
 void upload_slot_operators(pnop_ctx* c, int slot, const pnop::HostOps& h) {
     const size_t ns = (size_t)c->nslot;
     // v into the table of slot `at` (stride `stride` values, at least v.size())
-    auto put = [&](double*& dst, const std::vector<double>& v, size_t slots, size_t at, size_t stride = 0) {
+    auto put = [&](double*& dst, const auto& v, size_t slots, size_t at, size_t stride = 0) {
         stride = std::max(stride, v.size());
         if (!dst) dst = (double*)c->dalloc(std::max<size_t>(1, stride) * slots * sizeof(double));
         ck(cudaMemcpy(dst + at * stride, v.data(), v.size() * sizeof(double), cudaMemcpyHostToDevice), "upload");

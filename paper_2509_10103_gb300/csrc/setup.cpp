@@ -286,7 +286,7 @@ static double band_backward_error(const Band& A, const std::vector<double>& f, u
     return rmax / (amax * xmax + 1e-300);
 }
 
-static void scatter_factors(std::vector<double>& dst, int mat, int k, int nr, int ntile, int nc1,
+static void scatter_factors(RawVec& dst, int mat, int k, int nr, int ntile, int nc1,
                             const std::vector<double>& f) {
     for (int j = 0; j < nr; ++j)
         for (int e = 0; e < kBand; ++e) dst[fac_index(mat, k, j, e, nr, ntile, nc1)] = f[(size_t)j * kBand + e];
@@ -710,7 +710,7 @@ template <class F> static void parallel_k(int n, F&& fn) {
 // (matrix, table tile), so that a host thread writes whole tiles.  False when a
 // LU breaks down.
 template <class F, class E>
-static bool factor_tables(const HostOps& h, FixedTable& t, std::vector<double>& fac, std::vector<double>& facT,
+static bool factor_tables(const HostOps& h, FixedTable& t, RawVec& fac, RawVec& facT,
                           int nmat, F&& matrix, E&& each, double& worst) {
     const int nr = h.d.nr, nk = h.d.nk, nht = (nk + kTileX - 1) / kTileX;
     const FxShape shape = fx_shape(nr);
@@ -730,8 +730,8 @@ static bool factor_tables(const HostOps& h, FixedTable& t, std::vector<double>& 
         for (int j = 1; j <= kLo; ++j) col = std::max(col, std::fabs(A.get(j, 0) / A.get(0, 0)));
         if (std::isfinite(col))
             while (std::ldexp(col, -t.shift) > 1.0) ++t.shift;
-        t.direct.assign((size_t)nmat * nht * shape.tile, 0.0);
-        t.transposed.assign(t.direct.size(), 0.0);
+        t.direct.resize((size_t)nmat * nht * shape.tile);
+        t.transposed.resize(t.direct.size());
     }
     std::vector<double> err_t(16, 0.0), sum(16, 0.0), col(16, 0.0);
     std::vector<int> fail(16, 0), unfit(16, 0);
@@ -740,6 +740,8 @@ static bool factor_tables(const HostOps& h, FixedTable& t, std::vector<double>& 
         std::vector<double> f;
         Twist w;
         double growth = 0;
+        for (RawVec* v : {&t.direct, &t.transposed})
+            if (t.ok) std::fill_n(v->begin() + (size_t)item * shape.tile, shape.tile, 0.0);
         for (int k = k0; k < std::min(nk, k0 + kTileX) && !fail[th]; ++k) {
             const Band A = matrix(ma, kz(k));
             if (!band_lu(A, f, growth)) {
@@ -769,10 +771,12 @@ static bool factor_tables(const HostOps& h, FixedTable& t, std::vector<double>& 
     if (ok) return true;
     t = FixedTable{};
     const int nt = h.ntile;
-    fac.assign((size_t)nmat * nt * nr * kBand * kTileK, 0.0);
-    facT.assign(fac.size(), 0.0);
+    const size_t tile = (size_t)nr * kBand * kTileK;
+    fac.resize((size_t)nmat * nt * tile);
+    facT.resize(fac.size());
     parallel_k(nmat * nt, [&](int item, int) {
         const int ma = item / nt, k0 = item % nt * kTileK;
+        for (RawVec* v : {&fac, &facT}) std::fill_n(v->begin() + (size_t)item * tile, tile, 0.0);
         std::vector<double> f;
         double growth = 0;
         for (int k = k0; k < std::min(nk, k0 + kTileK); ++k) {

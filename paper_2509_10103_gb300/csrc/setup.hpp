@@ -6,6 +6,8 @@
 
 #include <complex>
 #include <string>
+#include <memory>
+#include <utility>
 #include <vector>
 
 namespace pnop {
@@ -80,10 +82,21 @@ constexpr double kFxBackward = 2e-15;
 constexpr int kFxMinRows = 21;    // smaller grids keep the FP64 solver
 constexpr int kFxMaxChunks = 96;  // chunks of a side the solver keeps units for (768 rows in all)
 constexpr int kFxMid = 49;        // words of a side's middle per k
+// Memory that its first writer, one of the threads that fill a table, touches first
+// (zeroing 170 MB of tables on one thread took a quarter of a 64x64x256 context's
+// factorisation)
+template <class T> struct RawAlloc : std::allocator<T> {
+    template <class U> struct rebind {
+        using other = RawAlloc<U>;
+    };
+    template <class U> void construct(U* p) { ::new ((void*)p) U; }
+    template <class U, class... A> void construct(U* p, A&&... a) { ::new ((void*)p) U(std::forward<A>(a)...); }
+};
+using RawVec = std::vector<double, RawAlloc<double>>;
 struct FixedTable {
     bool ok = false;
     int shift = 0;
-    std::vector<double> direct, transposed;
+    RawVec direct, transposed;
 };
 struct FxShape {
     int h, chunks[2], pad;  // rows of side 0, chunks of the sides, empty positions of side 1
@@ -132,7 +145,7 @@ struct HostOps {
     //   facHT/facPT (A^T x = b): U_{j-8..j-1,j}, 1/U_jj, L_{j+1..j+4,j}  (nc1 = kNc1Transposed)
     int ntile = 0;
     FixedTable fxH, fxP;
-    std::vector<double> facH, facHT, facP, facPT;
+    RawVec facH, facHT, facP, facPT;
     std::vector<double> phi, dphi;              // [M+1][nk][nr] pressure of a unit wall datum, its radial derivative
     std::vector<double> infl;                   // [nm][3][nr][nk] influence response, pre-scaled by -1/delta
     std::vector<double> fluxg;                  // [nr] flux response of mode (0,0)
