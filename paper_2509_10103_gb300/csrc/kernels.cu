@@ -687,7 +687,8 @@ __global__ void k_stage_div(Geo g, const double2* __restrict__ F, double2* __res
 // copy.  Each of the 2 kSK threads sweeps the real or the imaginary part of one
 // system (the matrices are real).  Terms are accumulated oldest first, so the
 // dependence from one row to the next is a single FMA.
-constexpr int kRC = 8;  // rows per staged chunk
+constexpr int kRC = 8;        // rows per staged chunk
+constexpr int kRegRows = 24;  // grids up to this many radial points keep FP64 Helmholtz columns in registers
 
 __device__ __forceinline__ void cp_async16(void* sm, const void* gm) {
     const unsigned a = (unsigned)__cvta_generic_to_shared(sm);
@@ -801,7 +802,7 @@ __global__ void __launch_bounds__(2 * kSK) k_band_solve(Geo g, const double* __r
         }
         __syncthreads();
     }
-    if (WALL && k0 + sy < g.nk) {  // wall partials of the tentative velocity (as in k_band_solve_x)
+    if (WALL && k0 + sy < g.nk) {  // wall partials of the tentative velocity (as in k_band_solve_reg)
         usub = moved(usub, off);
         const double* us = usub ? reinterpret_cast<const double*>(usub) + comp : nullptr;
         double* P = pw + ((((size_t)slot * 3 + v) * g.nm + im) * g.nk + (k0 + sy)) * 2 + comp;
@@ -834,6 +835,152 @@ __global__ void __launch_bounds__(2 * kSK) k_band_solve(Geo g, const double* __r
             val.y += a.y;
         }
         x[o] = val;
+    }
+}
+
+// The same two-sweep solve with each thread's column held in registers, for the
+// Helmholtz systems of grids of at most MAXR radial points, which the integer
+// solver below does not take.  The column stays in x[0..MAXR): the forward sweep
+// reads its lower neighbours and the backward sweep its upper ones straight from
+// registers (every index is a compile-time constant after unrolling), so no
+// shared-memory round trip sits on the dependent chain of a row; shared memory
+// holds only the staged coefficient rows.  Bound by that chain and the FP64 pipe.
+// The arithmetic and its order are those of k_band_solve: the results are the
+// same to the last bit (up to the sign of zero).
+template <int NL, int NU, bool DIAG1, int MAXR, bool WALL>
+__global__ void __launch_bounds__(2 * kSK) k_band_solve_reg(Geo g, const double* __restrict__ fac, size_t fac_stride,
+                                                      double2* __restrict__ X, const double2* __restrict__ add,
+                                                      int helm, int zero_row0, double* __restrict__ pw,
+                                                      const double2* __restrict__ usub) {
+    grid_dep_sync();
+    constexpr int NC1 = NL + (DIAG1 ? 1 : 0);
+    constexpr int NC2 = kB - NC1;
+    constexpr int NCM = NC1 > NC2 ? NC1 : NC2;
+    constexpr int MAXCH = MAXR / kRC;
+    static_assert(MAXR % kRC == 0, "whole chunks");
+    extern __shared__ __align__(16) unsigned char smem[];
+    double* Cb = reinterpret_cast<double*>(smem);  // [2][kRC][NCM][kSK]
+    int bi = blockIdx.x;
+    const int kb = bi % g.ntile;
+    bi /= g.ntile;
+    const int im = bi % g.nm, v = bi / g.nm;
+    const int m = im - g.M;
+    const int mv = helm ? (v == 0 ? m + 1 : (v == 1 ? m - 1 : m)) : m;
+    const int k0 = kb * kSK;
+    const size_t S = (size_t)g.nr * g.nm * g.nk;
+    const int slot = g.slot[blockIdx.y];
+    const size_t off = (size_t)slot * g.fs;
+    fac += (size_t)slot * fac_stride;
+    X += off;
+    add = moved(add, off);
+    const double* T1 = fac + ((size_t)abs(mv) * g.ntile + kb) * (size_t)g.nr * kB * kSK;
+    const double* T2 = T1 + (size_t)g.nr * NC1 * kSK;
+    const int tid = threadIdx.x, sy = tid % kSK, comp = tid / kSK;
+    const int nr = g.nr, nch = (nr + kRC - 1) / kRC;
+    const bool on = k0 + sy < g.nk;
+    // this thread's column: the real or imaginary part of system (v, m, k0 + sy)
+    const double* xs = reinterpret_cast<const double*>(X + (size_t)v * S) + comp;
+    double x[MAXR];
+#pragma unroll
+    for (int j = 0; j < MAXR; ++j) x[j] = (on && j < nr) ? xs[2 * sidx(g, j, im, k0 + sy)] : 0.0;
+    auto stage = [&](int t) {  // chunk t of the sweep sequence into buffer t & 1
+        if (t >= 2 * nch) return;
+        const bool fwd = t < nch;
+        const int c = fwd ? t : 2 * nch - 1 - t;
+        const int rows = min(kRC, nr - c * kRC);
+        const int nc = fwd ? NC1 : NC2;
+        const double* src = (fwd ? T1 : T2) + (size_t)c * kRC * nc * kSK;
+        double* dst = Cb + (size_t)(t & 1) * kRC * NCM * kSK;
+        const int nseg = rows * nc * (kSK / 2);
+        for (int i = tid; i < nseg; i += 2 * kSK) cp_async16(dst + 2 * i, src + 2 * i);
+    };
+    stage(0);
+    cp_async_commit();
+#pragma unroll
+    for (int t = 0; t < MAXCH; ++t) {
+        if (t < nch) {
+            stage(t + 1);
+            cp_async_commit();
+            cp_async_wait1();
+            __syncthreads();
+            const double* C = Cb + (size_t)(t & 1) * kRC * NCM * kSK + sy;
+#pragma unroll
+            for (int r = 0; r < kRC; ++r) {
+                const int j = t * kRC + r;
+                if (j < nr) {
+                    double val = x[j];
+                    const bool full = !(NL == 8 && j > 8);
+#pragma unroll
+                    for (int e = 0; e < NL; ++e) {
+                        const int jj = j - NL + e;  // w1[e] of k_band_solve: oldest first
+                        if (jj >= 0 && (full || e >= NL - 4)) val = fma(-C[(r * NC1 + e) * kSK], x[jj >= 0 ? jj : 0], val);
+                    }
+                    if (DIAG1) val *= C[(r * NC1 + NL) * kSK];
+                    x[j] = val;
+                }
+            }
+            __syncthreads();
+        }
+    }
+#pragma unroll
+    for (int c = MAXCH - 1; c >= 0; --c) {
+        if (c < nch) {
+            const int t = 2 * nch - 1 - c;
+            stage(t + 1);
+            cp_async_commit();
+            cp_async_wait1();
+            __syncthreads();
+            const double* C = Cb + (size_t)(t & 1) * kRC * NCM * kSK + sy;
+            constexpr int O = DIAG1 ? 0 : 1;
+#pragma unroll
+            for (int r = kRC - 1; r >= 0; --r) {
+                const int j = c * kRC + r;
+                if (j < nr) {
+                    double val = x[j];
+                    const bool full = !(NU == 8 && j >= 4);
+#pragma unroll
+                    for (int e = NU - 1; e >= 0; --e) {
+                        const int jj = j + 1 + e;  // w2[e] of k_band_solve: nearest first (0 beyond nr)
+                        if (jj < MAXR && (full || e < 4)) val = fma(-C[(r * NC2 + O + e) * kSK], x[jj < MAXR ? jj : 0], val);
+                    }
+                    if (!DIAG1) val *= C[(r * NC2) * kSK];
+                    x[j] = val;
+                }
+            }
+            __syncthreads();
+        }
+    }
+    if (!on) return;
+    if (WALL) {  // wall partials of the tentative velocity T^-1 x - usub, as in k_band_solve
+        const double* us = usub ? reinterpret_cast<const double*>(usub + off) + comp : nullptr;
+        double* P = pw + ((((size_t)slot * 3 + v) * g.nm + im) * g.nk + (k0 + sy)) * 2 + comp;
+        double acc = 0.0;
+        if (v < 2) {  // d0 . (x/2 - usub_r) over rows 0..8, d0 the wall row of D1 for u_r
+            const double* d0 = g.D1 + (size_t)par_idx(m + 1) * nr * kB + 4;
+#pragma unroll
+            for (int c = 0; c <= 8; ++c) {
+                double xv = 0.5 * x[c];
+                if (v == 0 && us) xv -= us[2 * sidx(g, c, im, k0 + sy)];
+                acc = fma(__ldg(d0 + c), xv, acc);
+            }
+            *P = acc;
+        } else if (m == 0 && k0 + sy == 0) {  // the mean mode's u_z: sum_j W_j (x - usub_z)
+#pragma unroll
+            for (int j = 0; j < MAXR; ++j)
+                if (j < nr) acc = fma(g.W[j], us ? x[j] - us[2 * (2 * S + sidx(g, j, im, 0))] : x[j], acc);
+            *P = acc;
+        }
+    }
+    double* xo = reinterpret_cast<double*>(X + (size_t)v * S) + comp;
+    const double* ad = add ? reinterpret_cast<const double*>(add + (size_t)v * S) + comp : nullptr;
+#pragma unroll
+    for (int j = 0; j < MAXR; ++j) {
+        if (j < nr) {
+            const size_t o = 2 * sidx(g, j, im, k0 + sy);
+            double val = (zero_row0 && j == 0) ? 0.0 : x[j];
+            if (ad) val += ad[o];
+            xo[o] = val;
+        }
     }
 }
 
@@ -2184,13 +2331,25 @@ static void launch_band_solve(const Geo& g, const double* fac, size_t fac_stride
         else go(k_band_solve_x<true, false>);
     }
     if (gd.nb) {
-        const size_t sm = (size_t)g.nr * kSK * sizeof(double2) + 2 * (size_t)kRC * 9 * kSK * sizeof(double);
+        const size_t coef = 2 * (size_t)kRC * 9 * kSK * sizeof(double), col = (size_t)g.nr * kSK * sizeof(double2);
+        // Columns in registers for the Helmholtz solves of grids of 17 to 20 points (24
+        // where a table does not fit) whose systems need a second wave of the
+        // shared-memory form's four blocks to an SM: at 20 points and 64x256 a stage
+        // takes 84.3 against 90.7 us, its transpose 93.7 against 107.2.  In one wave, and
+        // on smaller grids, that form is as fast or faster (20 points, 32x64: 62.8 against
+        // 65.3 us; 16 points, 96x256: 86.7 against 88.4).
+        const unsigned blocks = (unsigned)((helm ? 3 : 1) * g.nm * g.ntile) * gd.nb;
+        const bool reg = helm && g.nr > 16 && g.nr <= kRegRows && blocks > 152 * (227u * 1024u / (unsigned)(coef + col + 1024));
+        const size_t sm = coef + (reg ? 0 : col);
         auto go = [&](auto kernel) {
             smem_limit((const void*)kernel);
             const dim3 grid((unsigned)((helm ? 3 : 1) * g.nm * g.ntile), (unsigned)gd.nb);
             launch_serial(kernel, grid, 2 * kSK, sm, s, gd, fac, fac_stride, X, add, helm, zero_row0, pw, usub);
         };
-        if (!trans && pw) go(k_band_solve<4, 8, false, true>);
+        if (reg && !trans && pw) go(k_band_solve_reg<4, 8, false, kRegRows, true>);
+        else if (reg && !trans) go(k_band_solve_reg<4, 8, false, kRegRows, false>);
+        else if (reg) go(k_band_solve_reg<8, 4, true, kRegRows, false>);
+        else if (!trans && pw) go(k_band_solve<4, 8, false, true>);
         else if (!trans) go(k_band_solve<4, 8, false, false>);
         else go(k_band_solve<8, 4, true, false>);
     }
