@@ -1299,10 +1299,10 @@ __device__ __forceinline__ void solve_fixed(XSide& a, const int2* TX, int sh0, i
             a.ready();
             const int4* C = reinterpret_cast<const int4*>(a.buf[t & 1]) + kk;
             const int2* Cd = a.buf[t & 1] + kXR * 4 * kXK + kk;
-            // D^-1 y, at most 62 bits: 1/D is D' 2^(s - 60), s + 128 the low byte
-            // of D'; the rows of a chunk share s except in the first one
+            // D^-1 y, at most 62 bits: 1/D is D' 2^(s - 60); the rows of a chunk share
+            // s, two bits of s + 128 in each, but in the first one, where it is a byte
             long long z[kXR];
-            int mz = 0, mr[kXR], sr[kXR];
+            int mz = 0, mr[kXR], sr[kXR], shared = 0;
 #pragma unroll
             for (int r = 0; r < kXR; ++r) {
                 const int2 D = Cd[r * kXK];
@@ -1313,8 +1313,9 @@ __device__ __forceinline__ void solve_fixed(XSide& a, const int2* TX, int sh0, i
                 mr[r] = x_mag(x_split(z[r]));
                 mz |= mr[r];
                 sr[r] = D.x & 0xFF;
+                shared |= (D.x & 3) << (2 * r);
             }
-            int ez = Es[c] - 128 + sr[0], e = ez + (mz ? 63 - __clz(mz) : 31) - 59;
+            int ez = Es[c] - 128 + shared, e = ez + (mz ? 63 - __clz(mz) : 31) - 59;
             if (c == 0) {  // to a common unit
                 int top = kXZero;
 #pragma unroll

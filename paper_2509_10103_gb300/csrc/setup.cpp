@@ -594,11 +594,11 @@ static bool fx_write(FixedTable& tab, int mat, int k, int nht, const FxShape& f,
                 }
             }
         }
-        // 1/D = D' 2^(q - 60), D' of at most 62 bits with q + 128 as its low byte
-        // (the bits above are rounded for the byte to be part of the value).  The
-        // rows of a chunk of four share q except in the first chunk (the wall row).
-        // A row whose 1/D is more than 2^6 below the largest of its chunk would
-        // keep too few bits.
+        // 1/D = D' 2^(q - 60), D' of at most 62 bits.  The rows of a chunk of four share
+        // q, two bits of q + 128 being the lowest bits of each row's D', except in the
+        // first chunk (the wall row), where all eight are the low byte.  The bits above
+        // are rounded for these to be part of the value: 2^-54 of 1/D at most, down to
+        // rows 2^6 below the largest of their chunk.
         for (int p = 0; p < np - 4;) {
             const int end = p < 4 ? p + 1 : p + 4;
             int lo = 1 << 20, hi = -(1 << 20);
@@ -614,9 +614,12 @@ static bool fx_write(FixedTable& tab, int mat, int k, int nht, const FxShape& f,
             if (hi - lo > 6 || q < -127 || q > 127) return false;
             const double unit = std::ldexp(1.0, 60 - q);
             for (; p < end; ++p) {
-                const long long scaled = fx_round(t.d[s][p], unit), byte = q + 128;
+                const int bits = p < 4 ? 8 : 2, code = p < 4 ? q + 128 : ((q + 128) >> 2 * (p % 4)) & 3;
+                const long long scaled = fx_round(t.d[s][p], unit) - code + (1 << bits >> 1);
+                const long long c = ((scaled >> bits) << bits) + code;
+                const int low = (int)(unsigned)(c & 0xFFFFFFFFll);
                 const size_t o = base + f.out[s] + (size_t)(p / 4) * 20 * kTileX + (16 + p % 4) * kTileX + kk;
-                tab.direct[o] = tab.transposed[o] = fx_bits(((scaled - byte + 128) >> 8) * 256 + byte);
+                tab.direct[o] = tab.transposed[o] = fx_pair(low, (int)((c - low) >> 32));
             }
         }
         // S^-1 scaled by a power of two to row sums of at most 1, with 32 further

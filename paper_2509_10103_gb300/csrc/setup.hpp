@@ -58,8 +58,8 @@ constexpr int kNc1Transposed = kUp + 1;  // A^T x = b rows: U^T (8), 1/diag | L^
 // k) holds, a 16-byte read being two multipliers of one k:
 //   side 0 then side 1:  inward, [chunk][4][2][k][2] (positions p-4..p-1);
 //     outward, [chunk but the last]: [4][2][k][2] (positions p+1..p+4) and 1/D as
-//     [4][k], a 62-bit fixed-point number whose low byte is its exponent, shared
-//     by the rows of a chunk but in the first one; the side's half of S^-1 (or
+//     [4][k], a 62-bit fixed-point number whose lowest bits make up an exponent,
+//     shared by the rows of a chunk but in the first one; the side's half of S^-1 (or
 //     its transpose), [4][4][k][2] (own four, then the other side's four, in
 //     positions), the third digits of these entries, [4][4][k] (two 32-bit ones of
 //     one k each), and the exponent, [k];

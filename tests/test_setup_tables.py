@@ -4,7 +4,8 @@ program that checks what it builds against 113-bit arithmetic.
 - the pressure response to a unit wall datum, which the wall correction is made
   of, is rounded once (2^-52 of its largest value, however close to singular the
   matrix is);
-- the multipliers of the two-sided factorisation are rounded once, to 2^-58;
+- the multipliers of the two-sided factorisation are rounded once, to 2^-58, and
+  the reciprocals of its diagonal to 2^-54 of each;
 - the space that contexts reserve and report for the tables holds either form;
 - which grids the integer solver takes: every unstretched one of 21 to 768
   radial points at any Reynolds number, time step and length, and no other size;
@@ -91,7 +92,7 @@ int main(int argc, char** argv) {
         return worst <= std::ldexp(1.0, -52) ? 0 : 1;
     }
     if (what == "multipliers") {
-        double worst = 0;
+        double worst = 0, inverse = 0;
         for (int nr : {24, 41, 64}) {
             const HostOps h = build(nr, 2, 3, 25.0, 2000.0, 0.005, 0.0);
             const FxShape f = fx_shape(nr);
@@ -105,17 +106,28 @@ int main(int argc, char** argv) {
                         std::vector<std::vector<quad>> a(nr, std::vector<quad>(nr, 0));
                         for (int i = 0; i < nr; ++i)
                             for (int j = std::max(0, i - kLo); j <= std::min(nr - 1, i + kUp); ++j) a[i][j] = A.get(i, j);
-                        for (int c = 0; c < f.h - 4; ++c)  // side 0 is plain elimination from row 0
+                        for (int c = 0; c < f.h - 4; ++c) {  // side 0 is plain elimination from row 0
+                            const size_t out = (size_t)m * f.tile + f.out[0] + (size_t)(c / 4) * 20 * kTileX + 16 * kTileX + k;
+                            const long long d = units(t.direct[out + (size_t)(c % 4) * kTileX]);
+                            int code = (int)(d & 0xFF);
+                            if (c >= 4)
+                                for (int r = code = 0; r < 4; ++r)
+                                    code |= (int)(units(t.direct[out + (size_t)r * kTileX]) & 3) << 2 * r;
+                            const quad off = (quad)d * a[c][c] * (quad)std::ldexp(1.0, code - 128 - 60) - 1;
+                            inverse = std::max(inverse, (double)mag(off));
                             for (int i = c + 1; i <= c + 4; ++i) {
                                 const quad l = a[i][c] / a[c][c];
                                 for (int j = c; j < nr; ++j) a[i][j] -= l * a[c][j];
-                                const size_t at = (size_t)m * f.tile + f.in[0] + (((size_t)i * 2 + (c - i + 4) / 2) * kTileX + k) * 2 + (c - i + 4) % 2;
+                                const size_t at = (size_t)m * f.tile + f.in[0] +
+                                                  (((size_t)i * 2 + (c - i + 4) / 2) * kTileX + k) * 2 + (c - i + 4) % 2;
                                 const quad want = -l * (quad)std::ldexp(1.0, kFxBits - (c == 0 ? t.shift : 0));
                                 worst = std::max(worst, (double)mag((quad)units(t.direct[at]) - want));
                             }
+                        }
                     }
         }
-        std::printf("%.3g units\n", worst);
+        std::printf("%.3g units, 1/D %.3g\n", worst, inverse);
+        if (!(inverse <= std::ldexp(1.0, -54))) return 1;
         return worst <= 2.0 ? 0 : 1;  // one to nearest, one where the low digit is kept above -2^31
     }
     if (what == "grids") {
