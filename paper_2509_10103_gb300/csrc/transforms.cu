@@ -469,9 +469,9 @@ __device__ __forceinline__ int x_top(long long v) { return 64 - __clzll(v ^ (v >
 // points (FP64 arithmetic: 2e-16 to 6e-16, and up to 2e-12 where a small
 // component shared a packed column with a large one).  At most 80 registers:
 // 43.6 -> 41.9 us at 48x32x96, whose blocks are the smaller for it.
-// The fields fall into the groups u, w and (mode ZADJ) g; a group's input scale
-// is gs for k = 0 and gs hs for k > 0, hs a power of two (hsh its exponent),
-// and gs is part of the output scales o0, ok.
+// The fields fall into the groups u, w and (mode ZADJ) g; g's input scale is gs
+// for k = 0 and gs hs for k > 0, hs a power of two (hsh its exponent), and gs is
+// part of the output scales o0, ok.
 struct XScales {
     int hsh[3];
     double o0[6], ok[6];
@@ -1504,14 +1504,18 @@ static bool zpass2_any(const Geo& g, const T2* Y, T2* Z, const ZScales& sc, cons
 template <int MODE>
 static void zpass_fixed(const Geo& g, const double2* Y, double2* Z, const ZScales& sc, const int4* tw, cudaStream_t s) {
     constexpr int NPI = MODE == ZFWD ? 3 : 5, NG = MODE == ZFWD ? 2 : 3, NOUT = MODE == ZFWD ? 3 : 6;
+    // u and w come as they are; the cotangents (ZADJ) may have a scale, smaller by a
+    // power of two for k > 0, which every output of theirs is linear in
     XScales x{};
     double gs = 1.0;
-    for (int i = 0; i < NG; ++i) {
-        int e = 0;
-        if (std::frexp(sc.hk[3 * i] / sc.h0[3 * i], &e) != 0.5 || e > 1)
-            throw std::runtime_error("zpass: unsupported input scales");
-        x.hsh[i] = 1 - e;
-        gs *= sc.h0[3 * i];  // every output is linear in each of its groups; u and w are not scaled
+    for (int i = 0; i < 3 * NG; ++i) {
+        int e = 1;
+        bool ok = sc.h0[i] == sc.h0[i / 3 * 3] && sc.hk[i] == sc.hk[i / 3 * 3];
+        if (i < 6) ok = ok && sc.h0[i] == 1.0 && sc.hk[i] == 1.0;
+        else ok = ok && std::frexp(sc.hk[i] / sc.h0[i], &e) == 0.5 && e <= 1;
+        if (!ok) throw std::runtime_error("zpass: unsupported input scales");
+        x.hsh[i / 3] = 1 - e;
+        if (i == 6) gs = sc.h0[i];
     }
     for (int i = 0; i < NOUT; ++i) {
         x.o0[i] = sc.o0[i] * gs;
