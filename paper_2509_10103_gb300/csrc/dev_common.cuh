@@ -64,14 +64,6 @@ __device__ __forceinline__ double half_of(double x) {
     return __hiloint2double((int)h, (int)(small ? (lo >> 1) | (m << 31) : lo));
 }
 
-template <class T2> __device__ __forceinline__ T2 from_d(double2 v);
-template <> __device__ __forceinline__ double2 from_d<double2>(double2 v) { return v; }
-// The theta synthesis converts with the hardware (its FP64 pipe has room
-// between the loads), the theta analysis by integer operations (its FP64 pipe
-// also carries the additions of the base-flow terms): each measured fastest
-// that way on the 64x64x256 gradient.
-template <> __device__ __forceinline__ float2 from_d<float2>(double2 v) { return make_float2((float)v.x, (float)v.y); }
-__device__ __forceinline__ double2 to_d(double2 v) { return v; }
 __device__ __forceinline__ double2 to_d(float2 v) { return make_double2(f64_of(v.x), f64_of(v.y)); }
 
 __device__ __forceinline__ int par_idx(int m) { return m & 1; }  // 0 even, 1 odd (two's complement)
@@ -100,7 +92,7 @@ static inline unsigned nblk(size_t n, int bs) { return (unsigned)((n + bs - 1) /
 // the predecessor ends, instead of after a full launch round trip; it never
 // reads or writes memory before the wait, so stream order is kept.
 // launch_serial launches without that relaxation: the single-wave kernels
-// whose time depends on an even spread of their blocks over the SMs (the
+// whose time depends on an even spread of their blocks over the SMs (the FP64
 // banded solves) use it, so that all their blocks are placed on an idle GPU.
 __device__ __forceinline__ void grid_dep_sync() {
     asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -1,7 +1,9 @@
 // Spectral <-> physical transforms of the pseudo-spectral pipe-flow step
 // (Keuchel & Avila, Section 2.4): theta synthesis, the z pass with the
 // pointwise products of the nonlinear term, theta analysis.  3/2-padded grids,
-// hand-written shared-memory FFTs templated on FP64 or FP32.  Batched launches
+// hand-written FFTs in shared memory: in FP32 for the mixed precisions, in 64-bit
+// fixed point for the FP64 ones, but for the z pass of the continuous adjoint,
+// which is in FP64 there.  Batched launches
 // carry the batch entry in the grid's z dimension (with the field index for
 // the theta kernels) and offset spectral and physical buffers by its slot.
 #include "dev_common.cuh"
@@ -115,17 +117,17 @@ __device__ T2* fft_cols(T2* a, T2* b, int N, const T2* tw) {
     return a;
 }
 
-// spectral input value of a synthesis: fields stored in FP32 (FieldPtrs::inf)
-// are read as they are, FP64 fields converted to the transform precision
-template <class T2> __device__ __forceinline__ T2 from_f(float2 v);
-template <> __device__ __forceinline__ float2 from_f<float2>(float2 v) { return v; }
-template <> __device__ __forceinline__ double2 from_f<double2>(float2 v) { return to_d(v); }
-// an analysis result for an FP32 output field (FP64 transforms round it)
-__device__ __forceinline__ float2 to_f(float2 v) { return v; }
-__device__ __forceinline__ float2 to_f(double2 v) { return make_float2((float)v.x, (float)v.y); }
+// spectral input value of an FP32 synthesis: fields stored in FP32
+// (FieldPtrs::inf) are read as they are, FP64 fields converted (with the hardware,
+// whose FP64 pipe has room between the loads; the theta analysis converts by
+// integer operations, since its FP64 pipe also carries the additions of the
+// base-flow terms: each measured fastest that way on the 64x64x256 gradient)
 template <class T2>
 __device__ __forceinline__ T2 synth_in(const double2* src, const float2* srcf, size_t i) {
-    return srcf ? from_f<T2>(srcf[i]) : from_d<T2>(src[i]);
+    static_assert(std::is_same<T2, float2>::value, "FP64 fields take k_synth_x");
+    if (srcf) return srcf[i];
+    const double2 v = src[i];
+    return make_float2((float)v.x, (float)v.y);
 }
 
 // ------------------------------------------------------------------ theta synthesis
@@ -855,7 +857,7 @@ __global__ void k_anal_theta(Geo g, FieldPtrs f, const T2* __restrict__ Z, const
                 const T2 vm = res[(m > 0 ? g.nt - m : -m) * KB + kk];
                 v = mk<T2>((T)0.5 * (v.x + vm.x), (T)0.5 * (v.y - vm.y));
             }
-            dstf[o] = to_f(v);
+            dstf[o] = v;
             continue;
         }
         double2 v = to_d(res[(m < 0 ? m + g.nt : m) * KB + kk]);
@@ -1146,7 +1148,7 @@ __global__ void __launch_bounds__(kT2, sizeof(T2) == 8 ? 6 : 1) k_anal2(Geo g, F
                 if (k == 0) {
                     buf[n * KB + kk] = v[m1];
                 } else if (dstf) {
-                    dstf[(size_t)(m + g.M) * g.nk + k] = to_f(v[m1]);
+                    dstf[(size_t)(m + g.M) * g.nk + k] = v[m1];
                 } else {
                     const size_t o = (size_t)(m + g.M) * g.nk + k;
                     double2 x = to_d(v[m1]);
@@ -1166,7 +1168,7 @@ __global__ void __launch_bounds__(kT2, sizeof(T2) == 8 ? 6 : 1) k_anal2(Geo g, F
             if (dstf) {
                 using T = typename RealOf<T2>::T;
                 const T2 v = buf[(m < 0 ? m + N : m) * KB], vm = buf[(m > 0 ? N - m : -m) * KB];
-                dstf[(size_t)im * g.nk] = to_f(mk<T2>((T)0.5 * (v.x + vm.x), (T)0.5 * (v.y - vm.y)));
+                dstf[(size_t)im * g.nk] = mk<T2>((T)0.5 * (v.x + vm.x), (T)0.5 * (v.y - vm.y));
                 continue;
             }
             const double2 v = to_d(buf[(m < 0 ? m + N : m) * KB]);
@@ -1547,20 +1549,19 @@ void launch_zpass(const Geo& g, int mode, const T2* Y, T2* Z, const ZScales& sc_
         sc.fok[i] = (float)sc.ok[i];
     }
     const T2* t = tw_z<T2>(tw);
-    bool done = false;
     if constexpr (std::is_same<T2, double2>::value) {
-        done = mode != ZCADJ;
         if (mode == ZFWD) zpass_fixed<ZFWD>(g, Y, Z, sc, tw.z_x, s);
         else if (mode == ZADJ) zpass_fixed<ZADJ>(g, Y, Z, sc, tw.z_x, s);
-    }
-    if constexpr (std::is_same<T2, float2>::value)
-        done = mode == ZFWD ? zpass2_any<T2, ZFWD>(g, Y, Z, sc, t, s)
-                            : (mode == ZADJ ? zpass2_any<T2, ZADJ>(g, Y, Z, sc, t, s)
-                                            : zpass2_any<T2, ZCADJ>(g, Y, Z, sc, t, s));
-    if (!done) {
-        if (mode == ZFWD) zpass_stockham<T2, ZFWD>(g, Y, Z, sc, t, s);
-        else if (mode == ZADJ) zpass_stockham<T2, ZADJ>(g, Y, Z, sc, t, s);
         else zpass_stockham<T2, ZCADJ>(g, Y, Z, sc, t, s);
+    } else {
+        const bool done = mode == ZFWD ? zpass2_any<T2, ZFWD>(g, Y, Z, sc, t, s)
+                                       : (mode == ZADJ ? zpass2_any<T2, ZADJ>(g, Y, Z, sc, t, s)
+                                                       : zpass2_any<T2, ZCADJ>(g, Y, Z, sc, t, s));
+        if (!done) {
+            if (mode == ZFWD) zpass_stockham<T2, ZFWD>(g, Y, Z, sc, t, s);
+            else if (mode == ZADJ) zpass_stockham<T2, ZADJ>(g, Y, Z, sc, t, s);
+            else zpass_stockham<T2, ZCADJ>(g, Y, Z, sc, t, s);
+        }
     }
     check_launch("zpass");
 }
