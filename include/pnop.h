@@ -64,10 +64,15 @@ enum {
  *     the FP32 rate on this GPU.
  * Everything else (the radial banded solves, the influence and flux
  * corrections, the base flow, the stage combinations, energies and inner
- * products) stays FP64.  PNOP_FP64 (0) is FP64 throughout.  In every precision
- * the banded solves run in 64-bit block-floating integer arithmetic, which
- * rounds below FP64 arithmetic, where a grid's factors fit it (all unstretched
- * grids of 21 radial points or more), else in FP64. */
+ * products) stays FP64.  PNOP_FP64 (0) is FP64 throughout.
+ * FP64 values are held and returned in every case; two kinds of kernels compute
+ * them in 64-bit integers with shared exponents, with errors at or below the
+ * level of FP64 arithmetic: the banded solves (all precisions), where a grid's
+ * factors fit, as they do on unstretched grids of 21 to 768 radial points, else
+ * in FP64; and the transforms of contexts without PNOP_MIXED, but for the z
+ * transforms of the continuous adjoint.  A NaN or an infinity makes NaN of the
+ * whole radial column of its mode in such a solve, and of the values it reaches
+ * in such a transform; other modes and rows do not change. */
 enum { PNOP_FP64 = 0, PNOP_MIXED = 1, PNOP_DF = 2, PNOP_MIXED_DF = 3 };
 
 /* Grid.  nr radial points (>= 9); ntheta, nz nominal azimuthal/axial sizes,

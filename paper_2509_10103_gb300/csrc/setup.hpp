@@ -68,9 +68,9 @@ constexpr int kNc1Transposed = kUp + 1;  // A^T x = b rows: U^T (8), 1/diag | L^
 // The wall row of A (Dirichlet or Neumann) is not scaled like the others, so
 // column 0 of N is large: it is stored times 2^-shift and its value enters the
 // window times 2^shift.  The solver's 64-bit sums need sum |multiplier| <=
-// kFxRowSum in every row; on the unstretched grid the sums stay below 4.0 for
-// the pressure and 2.5 for the Helmholtz matrices (24 to 128 points, any Re dt);
-// wide one-sided stencils of stretched grids can exceed it (62 at stretch 0.1).
+// kFxRowSum in every row; on unstretched grids the sums are at most 4.0 (21 to 768
+// points, Re 1 to 1e5, dt 1e-5 to 1, lengths 0.5 to 1000); wide one-sided stencils
+// of stretched grids can exceed it (62 at stretch 0.1).
 constexpr int kTileX = 16;
 constexpr int kFxBits = 58;
 constexpr double kFxRowSum = 6.0;

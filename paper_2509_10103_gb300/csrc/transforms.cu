@@ -462,8 +462,8 @@ __device__ __forceinline__ int fx_unit(unsigned sum, int top, int bits) {
 __device__ __forceinline__ int x_top(long long v) { return 64 - __clzll(v ^ (v >> 63)); }  // |v| <= 2^top
 
 // The z pass in fixed point: contract of k_zpass (FP64), any length.  Bound by
-// integer issue and its barriers (44% of the warps' slots in use at 64x64x256);
-// 828 -> 207 us forward and 1308 -> 334 us adjoint against the FP64 Stockham
+// integer issue and its barriers (35% of the warps' slots in use at 64x64x256);
+// 828 -> 208 us forward and 1308 -> 341 us adjoint against the FP64 Stockham
 // kernel, 73 and 108 FP64 instructions a point at 77 cycles.  Every field has a
 // unit of its own (the components of u and of w differ by orders of magnitude
 // in streaky flows), and every output one from the larger of its two products:
@@ -689,10 +689,11 @@ __global__ void __launch_bounds__(256, 3)
 }
 
 // The theta transforms in fixed point, any length: contract of k_synth_theta and
-// k_anal_theta (FP64).  206 -> 74 us (synthesis) and 158 -> 64 us (analysis) at
-// 64x64x256 against the FP64 two-pass kernels.  A block takes KB columns k of one (field, j), all in one
-// unit (the z pass sums over k, so a column far below its neighbours does not
-// count there).  Rows of `in` values from memory into `raw`, and the unit in
+// k_anal_theta (FP64).  206 -> 68 us (synthesis) and 158 -> 69 us (analysis) at
+// 64x64x256 against the FP64 two-pass kernels.  A block takes KB columns k of one
+// (field, j), all in one unit (the z pass sums over k, so a column far below its
+// neighbours does not count there: on spectra falling as e^-k/4 to e^-k the error
+// of every k is 5 to 50 times below that of FP64 transforms).  Rows of `in` values from memory into `raw`, and the unit in
 // which the magnitudes of every column sum to less than 2^61; bad: infinities or NaN.
 template <int KB, class F>
 __device__ __forceinline__ int fx_columns(int rows, int kw, double2* raw, F&& load, int* top_sh, unsigned* sum_sh, bool& bad) {
@@ -1389,6 +1390,9 @@ static void anal2(const Geo& g, const FieldPtrs& f, int nfield, const T2* Z, con
 
 // columns per block of the fixed-point theta kernels: about 50 KB of shared
 // memory, 128 to 256 contiguous bytes per row
+// (64x64x256: synthesis 67 us at 16, 73 at 8, 76 at 4, analysis 57, 59, 54; 48x48x128: 26,
+// 28, 29 and 24, 23, 20; 48x32x96: 18, 18, 16 and 14, 14, 12; 64x96x128, 144 points: 67, 67, 78
+// and 50, 53, 53; 48x128x64, 192 points: 39, 34, 39 and 29, 29, 27)
 static int theta_kx(const Geo& g) { return g.nt <= 96 && g.nk > 8 ? 16 : (g.nt <= 192 ? 8 : 4); }
 template <int KB> static size_t theta_sx(const Geo& g) { return (size_t)(2 * g.nt * KB + g.nt) * sizeof(double2); }
 static unsigned theta_tx(const Geo& g, int kb) {
