@@ -1011,8 +1011,8 @@ __global__ void __launch_bounds__(2 * kSK) k_band_solve_reg(Geo g, const double*
 // pairs holding the real and imaginary parts; multipliers stream through the
 // warp's own shared memory with cp.async.  The two warps meet once, at the middle.
 // Measured against the FP64 kernels that served these solves before (64x64x256,
-// ncu): pressure 36.8 -> 24.5 us, Helmholtz with the wall partials 71.2 -> 51.2
-// us, the transposed pair 37.5 + 74.8 -> 74 us together; at 32x32x64 25.5 -> 14.6
+// ncu): pressure 36.8 -> 25.0 us, Helmholtz with the wall partials 71.2 -> 51.0
+// us, the transposed pair 37.5 + 74.8 -> 76 us together; at 32x32x64 25.5 -> 14.9
 // us per solve.  The errors of a whole stage against 113-bit arithmetic are half
 // (median, smooth fields) to a tenth (largest) of the FP64 kernels'.  Half as many rows per FP64 chain (the same sweeps in FP64, two-
 // sided) measured 33 and 96 us, and tiles split between the integer and the FP64
